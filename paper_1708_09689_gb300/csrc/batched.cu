@@ -173,9 +173,7 @@ __global__ void __launch_bounds__(256) kpm_batched_kernel(const __grid_constant_
                                       const Blk<T, VPT>& xp, const Blk<T, VPT>& ax, const Blk<T, VPT>& bx,
                                       const Blk<T, VPT>& ay, const Blk<T, VPT>& by,
                                       const Blk<T, VPT>* yi, Blk<T, VPT>& yn) {
-                                    Blk<T, VPT> S, D;
-                                    ti_axes(xm, xp, ax, bx, ay, by, S, D);
-                                    ti_combine_core(cf, Vs, xc, S, D, yi, yn);
+                                    ti_update(cf, Vs, xm, xc, xp, ax, bx, ay, by, yi, yn);
                                     if constexpr (decltype(with_delta)::value) ti_add_delta(L.g, cf, xc, yn);
                                   },
                                   [&](int64_t s, const Blk<T, VPT>& xc, Blk<T, VPT>& yn) {

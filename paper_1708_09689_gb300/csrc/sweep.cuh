@@ -766,6 +766,87 @@ __device__ __forceinline__ void ti_combine(const VecCoef<T, VPT>& cf, T Vs, cons
   if (g.has_delta) ti_add_delta(g, cf, xc, yn);
 }
 
+// The hopping sum T = Gamma^1 S + sum_j (-i Gamma^{j+1}) d_j in complex128.  Every bond
+// matrix Gamma^1 -+ i Gamma^{j+1} has rank 2: a neighbour enters through two projected
+// components h, and the two others are h again up to a sign or a factor +-i.  With a the
+// neighbour at n - e_j and b the one at n + e_j,
+//   z: a -> (h0, -h0, h1, -h1),    h = (a0 + a1, a2 + a3);    b -> (g0, g0, g1, g1),     g = (b0 - b1, b2 - b3)
+//   x: a -> (h0, h1, h1, -h0),     h = (a0 + a3, a2 - a1);    b -> (g0, -g1, g1, g0),    g = (b0 - b3, b2 + b1)
+//   y: a -> (h0, -ih1, h1, -ih0),  h = (a0 - ia3, a2 - ia1);  b -> (g0, ig1, g1, ig0),   g = (b0 + ib3, b2 + ib1)
+// which takes 64 real additions where S, D and their combination take 88.
+template <int VPT>
+__device__ __forceinline__ void ti_hop(const Blk<double, VPT>& zm, const Blk<double, VPT>& zp,
+                                       const Blk<double, VPT>& xm, const Blk<double, VPT>& xp,
+                                       const Blk<double, VPT>& ym, const Blk<double, VPT>& yp,
+                                       Blk<double, VPT>& H) {
+  using cd = cplx<double>;
+  auto addi = [](cd a, cd b) { return cd{a.re - b.im, a.im + b.re}; };  // a + i b
+  auto subi = [](cd a, cd b) { return cd{a.re + b.im, a.im - b.re}; };  // a - i b
+#pragma unroll
+  for (int v = 0; v < VPT; ++v) {
+    cd h0 = cadd(zm.v[0][v], zm.v[1][v]), h1 = cadd(zm.v[2][v], zm.v[3][v]);
+    cd g0 = csub(zp.v[0][v], zp.v[1][v]), g1 = csub(zp.v[2][v], zp.v[3][v]);
+    cd t0 = cadd(h0, g0), t1 = csub(g0, h0), t2 = cadd(h1, g1), t3 = csub(g1, h1);
+    h0 = cadd(xm.v[0][v], xm.v[3][v]);
+    h1 = csub(xm.v[2][v], xm.v[1][v]);
+    g0 = csub(xp.v[0][v], xp.v[3][v]);
+    g1 = cadd(xp.v[2][v], xp.v[1][v]);
+    t0 = cadd(t0, cadd(h0, g0));
+    t1 = cadd(t1, csub(h1, g1));
+    t2 = cadd(t2, cadd(h1, g1));
+    t3 = cadd(t3, csub(g0, h0));
+    h0 = subi(ym.v[0][v], ym.v[3][v]);
+    h1 = subi(ym.v[2][v], ym.v[1][v]);
+    g0 = addi(yp.v[0][v], yp.v[3][v]);
+    g1 = addi(yp.v[2][v], yp.v[1][v]);
+    H.v[0][v] = cadd(t0, cadd(h0, g0));
+    H.v[1][v] = addi(t1, csub(g1, h1));
+    H.v[2][v] = cadd(t2, cadd(h1, g1));
+    H.v[3][v] = addi(t3, csub(g0, h0));
+  }
+}
+
+// y_new of one TI site from the blocks around it (Delta terms aside).  complex64 folds S and
+// D (ti_axes, ti_combine_core).  complex128 is bound by the fp64 pipe of this part (1/64 of
+// the fp32 rate: two lanes per SM), so it takes the projected hopping sum and the shortest
+// update: with gamma = -1 (every recurrence sweep after the first) y_new = kt T + (d x - y_in)
+// in two fused operations a part.  100 fp64 operations per site and vector with two dot
+// products, from 133; the KPM sweep of a 128x128x64 lattice at R = 8 takes 2.22 ms, from 2.43
+// (the z-march's eight warps do not keep the pipe busy all the time: about 75 % of its rate).
+template <typename T, int VPT>
+__device__ __forceinline__ void ti_update(const VecCoef<T, VPT>& cf, T Vs, const Blk<T, VPT>& zm,
+                                          const Blk<T, VPT>& xc, const Blk<T, VPT>& zp, const Blk<T, VPT>& xm,
+                                          const Blk<T, VPT>& xp, const Blk<T, VPT>& ym, const Blk<T, VPT>& yp,
+                                          const Blk<T, VPT>* yi, Blk<T, VPT>& yn) {
+  if constexpr (sizeof(T) == 8) {
+    Blk<T, VPT> H;
+    ti_hop(zm, zp, xm, xp, ym, yp, H);
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) {
+      const T dp = fma(cf.alpha[v], Vs, cf.am[v] - cf.ab[v]), dm = fma(cf.alpha[v], Vs, -cf.am[v] - cf.ab[v]);
+      const bool minus = cf.gamma[v] == T(-1);
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        const T dd = (o & 1) ? dm : dp;
+        const cplx<T> x = xc.v[o][v];
+        cplx<T> t;
+        if (yi == nullptr) {
+          t = {dd * x.re, dd * x.im};
+        } else if (minus) {
+          t = {fma(dd, x.re, -yi->v[o][v].re), fma(dd, x.im, -yi->v[o][v].im)};
+        } else {
+          t = {fma(cf.gamma[v], yi->v[o][v].re, dd * x.re), fma(cf.gamma[v], yi->v[o][v].im, dd * x.im)};
+        }
+        yn.v[o][v] = {fma(cf.kt[v], H.v[o][v].re, t.re), fma(cf.kt[v], H.v[o][v].im, t.im)};
+      }
+    }
+  } else {
+    Blk<T, VPT> S, D;
+    ti_axes(zm, zp, xm, xp, ym, yp, S, D);
+    ti_combine_core(cf, Vs, xc, S, D, yi, yn);
+  }
+}
+
 template <typename T, int VPT, bool NC, int DEPTH, int NBUF, class Site, class Combine, class Emit>
 __device__ __forceinline__ void ti_march(const Geometry& g, const T* __restrict__ X,
                                          const T* __restrict__ Yin, int R, int rc, int64_t col,
@@ -918,9 +999,8 @@ __global__ void __launch_bounds__(256, (VPT == 1 && sizeof(T) == 4) ? 2 : 1) ti_
                                const Blk<T, VPT>& xp, const Blk<T, VPT>& ax, const Blk<T, VPT>& bx,
                                const Blk<T, VPT>& ay, const Blk<T, VPT>& by, const Blk<T, VPT>* yi,
                                Blk<T, VPT>& yn) {
-                             Blk<T, VPT> S, D;
-                             ti_axes(xm, xp, ax, bx, ay, by, S, D);
-                             ti_combine(cf, Vs, xc, S, D, yi, yn, p.g);
+                             ti_update(cf, Vs, xm, xc, xp, ax, bx, ay, by, yi, yn);
+                             if (p.g.has_delta) ti_add_delta(p.g, cf, xc, yn);
                            },
                            [&](int64_t s, const Blk<T, VPT>& xc, Blk<T, VPT>& yn) {
                              const int64_t sites[4] = {s, s, s, s};
@@ -937,7 +1017,7 @@ __global__ void __launch_bounds__(256, (VPT == 1 && sizeof(T) == 4) ? 2 : 1) ti_
 // TI sweep marching along x (for lattices whose z extent is short): a thread
 // keeps sites x-1, x, x+1 of its line (y, z) in registers and reads the y and
 // z neighbours, which the threads of neighbouring lines load, from L1/L2.  The
-// neighbours enter ti_axes in the same order as in the z-march (z pair, x
+// neighbours enter ti_update in the same order as in the z-march (z pair, x
 // pair, y pair), so the result equals the z-marching sweep's bit for bit.
 // Units: groups of blockDim / C lines (y fastest) times x-segments of p.zslab
 // sites (whole lines when p.zslab >= Lx).
@@ -980,15 +1060,15 @@ __global__ void __launch_bounds__(256) ti_sweep_xmarch(const __grid_constant__ S
       const int64_t s = base + x;
       const int64_t q = nbr_plus(x, x, Lx, g.per[0], 1);
       if (q >= 0) load_at<T, VPT, true>(at(base + q), R, xp); else zero_blk(xp);
-      Blk<T, VPT> yi, za, zb, ya, yb, S, D, yn;
+      Blk<T, VPT> yi, za, zb, ya, yb, yn;
       if (Yin != nullptr) load_at<T, VPT, false>(Yin + s * SS + cofs, R, yi);
       if (lzm >= 0) load_at<T, VPT, true>(at(lzm + x), R, za); else zero_blk(za);
       if (lzp >= 0) load_at<T, VPT, true>(at(lzp + x), R, zb); else zero_blk(zb);
       if (lym >= 0) load_at<T, VPT, true>(at(lym + x), R, ya); else zero_blk(ya);
       if (lyp >= 0) load_at<T, VPT, true>(at(lyp + x), R, yb); else zero_blk(yb);
       const T Vs = site_potential_t<T>(g, s);
-      ti_axes(za, zb, xm, xp, ya, yb, S, D);
-      ti_combine(cf, Vs, xc, S, D, Yin != nullptr ? &yi : nullptr, yn, g);
+      ti_update(cf, Vs, za, xc, zb, xm, xp, ya, yb, Yin != nullptr ? &yi : nullptr, yn);
+      if (g.has_delta) ti_add_delta(g, cf, xc, yn);
       const int64_t sites[4] = {s, s, s, s};
       epilogue<T, VPT, FEAT>(p, s, rc, xc, yn, dacc, sites, yi);
       xm = xc;
