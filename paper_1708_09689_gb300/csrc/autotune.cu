@@ -161,11 +161,11 @@ extern "C" int pvsc_autotune_op(pvsc_lattice* lat, int R, int prec, int op, pvsc
     p.cz_re = -0.1;
     PVSC_CUDA_TRY(cudaMemsetAsync(work, 0, kWorkHeader, st));
     auto one = [&]() -> int {
-      if (op == PVSC_OP_KPM) return launch_sweep(lat, prec, F_DOTS, p, st);
+      if (op == PVSC_OP_KPM) return launch_sweep(lat, prec, F_KPM, p, st);
       if (op == PVSC_OP_APPLY) return launch_sweep(lat, prec, 0, p, st);
       if (int r = launch_sweep(lat, prec, F_ACC, p, st)) return r;
-      if (int r = launch_sweep(lat, prec, 0, p, st)) return r;
-      return launch_sweep(lat, prec, 0, p, st);
+      if (int r = launch_sweep(lat, prec, F_REC, p, st)) return r;
+      return launch_sweep(lat, prec, F_REC, p, st);
     };
     if (int r = one()) return r;
     // the best of three trials of three repetitions each: shapes a few per cent

@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(256) kpm_batched_kernel(const __grid_constant_
                                       const Blk<T, VPT>& xp, const Blk<T, VPT>& ax, const Blk<T, VPT>& bx,
                                       const Blk<T, VPT>& ay, const Blk<T, VPT>& by,
                                       const Blk<T, VPT>* yi, Blk<T, VPT>& yn) {
-                                    ti_update(cf, Vs, xm, xc, xp, ax, bx, ay, by, yi, yn);
+                                    ti_update<true>(cf, Vs, xm, xc, xp, ax, bx, ay, by, yi, yn);
                                     if constexpr (decltype(with_delta)::value) ti_add_delta(L.g, cf, xc, yn);
                                   },
                                   [&](int64_t s, const Blk<T, VPT>& xc, Blk<T, VPT>& yn) {
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(256) kpm_batched_kernel(const __grid_constant_
           if (L.g.has_delta) march(std::true_type{});
           else march(std::false_type{});
         }
-        dacc.flush();
+        dacc.flush(2);
         // fixed-order block reduction to one row of partials for this unit
 #pragma unroll
         for (int d = 0; d < 2; ++d)

@@ -304,6 +304,7 @@ __device__ __forceinline__ void finish_dots(const Sweep& p) {
   for (int q = warp; q < kNumDots * p.R; q += nwarps) {
     const int d = q / p.R, r = q % p.R;
     if (!((p.dot_flags >> (d == 0 ? 0 : (d == 3 ? 2 : 1))) & 1)) continue;
+    if ((p.dot_mode == 1 || p.dot_mode == 2) && d > 1) continue;  // a KPM step reads the first two
     double s = 0.0;
     for (int b = lane; b < nb; b += 32) s += __ldcg(p.partials + (size_t)b * kNumDots * p.R + q);
 #pragma unroll
@@ -329,14 +330,16 @@ __device__ __forceinline__ void finish_dots(const Sweep& p) {
   if (threadIdx.x == 0) *p.counter = 0u;
 }
 
-template <int VPT, int MAXW = kMaxThreads / 32>
+// ND: the dots this sweep forms (a KPM step: the first two; the others' rows stay unwritten
+// and finish_dots does not read them).
+template <int VPT, int MAXW = kMaxThreads / 32, int ND = kNumDots>
 __device__ void reduce_dots(const Sweep& p, double (&acc)[kNumDots][VPT]) {
-  __shared__ double sm[MAXW][kNumDots][VPT][32];  // [warp][dot][v][lane]
+  __shared__ double sm[MAXW][ND][VPT][32];  // [warp][dot][v][lane]
   const int C = p.C;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nwarps = blockDim.x >> 5;
 #pragma unroll
-  for (int d = 0; d < kNumDots; ++d)
+  for (int d = 0; d < ND; ++d)
 #pragma unroll
     for (int v = 0; v < VPT; ++v) {
       double s = acc[d][v];
@@ -349,7 +352,7 @@ __device__ void reduce_dots(const Sweep& p, double (&acc)[kNumDots][VPT]) {
     const int stride = C < 32 ? 1 : C / 32;  // warps that carry chunk t
     const int w0 = C < 32 ? 0 : t / 32;
     const int l = C < 32 ? t : t % 32;
-    for (int d = 0; d < kNumDots; ++d)
+    for (int d = 0; d < ND; ++d)
       for (int v = 0; v < VPT; ++v) {
         double s = 0.0;
         for (int w = w0; w < nwarps; w += stride) s += sm[w][d][v][l];

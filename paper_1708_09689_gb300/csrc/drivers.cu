@@ -406,7 +406,7 @@ static int run_series(const pvsc_lattice* lat, int R, int prec, const void* x, v
     p.x = cur;
     p.yin = prev;
     p.yout = last ? nullptr : out;
-    int feat = 0;
+    int feat = F_REC;
     if (plan[j] > 0) {
       set_acc(j, ACC_ADD | (last ? ACC_FINAL : 0), plan[j]);
       feat = F_ACC;
@@ -462,7 +462,7 @@ int kpm_enqueue(const pvsc_lattice* lat, int R, int prec, const void* r0, uint64
   p.yin = nullptr;
   p.yout = wb;
   p.dot_mode = 1;
-  if (int rc = launch_sweep_shape(lat, prec, F_DOTS, p, sh, cs)) return rc;
+  if (int rc = launch_sweep_shape(lat, prec, F_KPM, p, sh, cs)) return rc;
   const void* prev = x0;
   void* cur = wb;
   const int nsteps = (M + 1) / 2;
@@ -501,7 +501,7 @@ int kpm_enqueue(const pvsc_lattice* lat, int R, int prec, const void* r0, uint64
     p.yin = prev;
     p.yout = out;
     p.kpm_k = k;
-    if (int rc = launch_sweep_shape(lat, prec, F_DOTS, p, sh, cs)) return rc;
+    if (int rc = launch_sweep_shape(lat, prec, F_KPM, p, sh, cs)) return rc;
     prev = cur;
     cur = out;
   }
@@ -762,7 +762,7 @@ int pvsc_kpm_sweeps(const pvsc_lattice* lat, int R, int prec, int k_begin, int k
     p.yout = other;
     p.dot_mode = k == 0 ? 1 : 2;
     p.kpm_k = k;
-    if (int rc = launch_sweep(lat, prec, F_DOTS, p, st)) return rc;
+    if (int rc = launch_sweep(lat, prec, F_KPM, p, st)) return rc;
   }
   return PVSC_OK;
 }
@@ -881,7 +881,7 @@ int pvsc_cheb_adjoint_step(const pvsc_lattice* lat, int R, int prec, const void*
     p.x = Wk(k - 1);
     p.yin = k == 1 ? nullptr : Wk(k - 2);
     p.yout = Wk(k);
-    if (int rc = launch_sweep(lat, prec, 0, p, st)) return rc;
+    if (int rc = launch_sweep(lat, prec, F_REC, p, st)) return rc;
   }
   // u_M = sigma_M G, grad += (f_{M-1}/a) Re conj(u_M) w_{M-1}
   {

@@ -20,9 +20,19 @@
 
 namespace pvsc {
 
-// F_DOTS: the dot products selected at run time by Sweep::dot_flags.
-enum Feat { F_DOTS = 1, F_Z = 2, F_ACC = 4, F_ADJ = 8 };
-__host__ __device__ constexpr bool has_dots(int feat) { return (feat & F_DOTS) != 0; }
+// F_DOTS: the dot products selected at run time by Sweep::dot_flags.  F_KPM: the two dot
+// products of a KPM step, <x|x> and Re<y|x>, alone.  F_REC: a plain recurrence sweep.
+// The recurrences (F_KPM, F_REC, F_ACC, F_ADJ) have gamma = -1 wherever they have a y_in, which
+// complex128 sweeps take at compile time: a test of gamma or of the flags at run time becomes
+// predicated fp64 instructions, which occupy the fp64 pipe also where they are switched off
+// (140 fp64-pipe instructions per site and vector counted in a KPM sweep, 100 needed).  F_KPM
+// against F_DOTS, KPM sweep: complex128 128x128x64, R = 8 2.22 -> 1.74 ms; complex64 256x256x64,
+// R = 8 (kernel 7) 514 -> 497 us; 101x87x53, R = 4 (z-march) 77.5 -> 68.0 us; Weyl 256x32x32,
+// R = 16 (flat) 65.6 -> 56.2 us.
+enum Feat { F_DOTS = 1, F_Z = 2, F_ACC = 4, F_ADJ = 8, F_KPM = 16, F_REC = 32 };
+__host__ __device__ constexpr bool has_dots(int feat) { return (feat & (F_DOTS | F_KPM)) != 0; }
+__host__ __device__ constexpr int num_dots(int feat) { return (feat & F_KPM) != 0 ? 2 : kNumDots; }
+__host__ __device__ constexpr bool is_recurrence(int feat) { return (feat & (F_KPM | F_REC | F_ACC | F_ADJ)) != 0; }
 
 // 16-byte vector of two 8-byte elements: complex128 (re, im) or the fixed-point pair
 template <typename T> struct Pair16 { using type = double2; };
@@ -224,12 +234,13 @@ struct DotAcc {
       s[k][v] = t;
     }
   }
-  __device__ __forceinline__ void flush() {
+  __device__ __forceinline__ void flush(int nd = kNumDots) {
     if constexpr (sizeof(T) == 4) {
 #pragma unroll
       for (int k = 0; k < kNumDots; ++k)
 #pragma unroll
         for (int v = 0; v < VPT; ++v) {
+          if (k >= nd) continue;
           d[k][v] += (double)s[k][v] + (double)c[k][v];
           s[k][v] = T(0);
           c[k][v] = T(0);
@@ -533,19 +544,20 @@ __device__ __forceinline__ void epilogue(const Sweep& p, int64_t s, int rc, cons
     // per-site products in T, accumulated per thread (compensated for fp32)
 #pragma unroll
     for (int v = 0; v < VPT; ++v) {
+      constexpr bool KPM = (FEAT & F_KPM) != 0;
       T xx = 0, xyr = 0, xyi = 0, yy = 0;
 #pragma unroll
       for (int o = 0; o < 4; ++o) {
         const cplx<T> a = xc.v[o][v], b = yn.v[o][v];
         xx = fma(a.re, a.re, fma(a.im, a.im, xx));
         xyr = fma(b.re, a.re, fma(b.im, a.im, xyr));
-        if (p.dot_flags & 2) xyi = fma(b.re, a.im, fma(-b.im, a.re, xyi));
-        if (p.dot_flags & 4) yy = fma(b.re, b.re, fma(b.im, b.im, yy));
+        if (!KPM && (p.dot_flags & 2)) xyi = fma(b.re, a.im, fma(-b.im, a.re, xyi));
+        if (!KPM && (p.dot_flags & 4)) yy = fma(b.re, b.re, fma(b.im, b.im, yy));
       }
       dacc.add(0, v, xx);
       dacc.add(1, v, xyr);
-      if (p.dot_flags & 2) dacc.add(2, v, xyi);
-      if (p.dot_flags & 4) dacc.add(3, v, yy);
+      if (!KPM && (p.dot_flags & 2)) dacc.add(2, v, xyi);
+      if (!KPM && (p.dot_flags & 4)) dacc.add(3, v, yy);
     }
   }
 }
@@ -774,72 +786,75 @@ __device__ __forceinline__ void ti_combine(const VecCoef<T, VPT>& cf, T Vs, cons
 //   x: a -> (h0, h1, h1, -h0),     h = (a0 + a3, a2 - a1);    b -> (g0, -g1, g1, g0),    g = (b0 - b3, b2 + b1)
 //   y: a -> (h0, -ih1, h1, -ih0),  h = (a0 - ia3, a2 - ia1);  b -> (g0, ig1, g1, ig0),   g = (b0 + ib3, b2 + ib1)
 // which takes 64 real additions where S, D and their combination take 88.
-template <int VPT>
-__device__ __forceinline__ void ti_hop(const Blk<double, VPT>& zm, const Blk<double, VPT>& zp,
-                                       const Blk<double, VPT>& xm, const Blk<double, VPT>& xp,
-                                       const Blk<double, VPT>& ym, const Blk<double, VPT>& yp,
-                                       Blk<double, VPT>& H) {
-  using cd = cplx<double>;
-  auto addi = [](cd a, cd b) { return cd{a.re - b.im, a.im + b.re}; };  // a + i b
-  auto subi = [](cd a, cd b) { return cd{a.re + b.im, a.im - b.re}; };  // a - i b
+__device__ __forceinline__ cplx<double> caddi(cplx<double> a, cplx<double> b) { return {a.re - b.im, a.im + b.re}; }
+__device__ __forceinline__ cplx<double> csubi(cplx<double> a, cplx<double> b) { return {a.re + b.im, a.im - b.re}; }
+
+__device__ __forceinline__ void hop_z_init(const Blk<double, 1>& a, const Blk<double, 1>& b, Blk<double, 1>& H) {
+  const cplx<double> h0 = cadd(a.v[0][0], a.v[1][0]), h1 = cadd(a.v[2][0], a.v[3][0]);
+  const cplx<double> g0 = csub(b.v[0][0], b.v[1][0]), g1 = csub(b.v[2][0], b.v[3][0]);
+  H.v[0][0] = cadd(h0, g0);
+  H.v[1][0] = csub(g0, h0);
+  H.v[2][0] = cadd(h1, g1);
+  H.v[3][0] = csub(g1, h1);
+}
+
+__device__ __forceinline__ void hop_x_add(const Blk<double, 1>& a, const Blk<double, 1>& b, Blk<double, 1>& H) {
+  const cplx<double> h0 = cadd(a.v[0][0], a.v[3][0]), h1 = csub(a.v[2][0], a.v[1][0]);
+  const cplx<double> g0 = csub(b.v[0][0], b.v[3][0]), g1 = cadd(b.v[2][0], b.v[1][0]);
+  H.v[0][0] = cadd(H.v[0][0], cadd(h0, g0));
+  H.v[1][0] = cadd(H.v[1][0], csub(h1, g1));
+  H.v[2][0] = cadd(H.v[2][0], cadd(h1, g1));
+  H.v[3][0] = cadd(H.v[3][0], csub(g0, h0));
+}
+
+__device__ __forceinline__ void hop_y_add(const Blk<double, 1>& a, const Blk<double, 1>& b, Blk<double, 1>& H) {
+  const cplx<double> h0 = csubi(a.v[0][0], a.v[3][0]), h1 = csubi(a.v[2][0], a.v[1][0]);
+  const cplx<double> g0 = caddi(b.v[0][0], b.v[3][0]), g1 = caddi(b.v[2][0], b.v[1][0]);
+  H.v[0][0] = cadd(H.v[0][0], cadd(h0, g0));
+  H.v[1][0] = caddi(H.v[1][0], csub(g1, h1));
+  H.v[2][0] = cadd(H.v[2][0], cadd(h1, g1));
+  H.v[3][0] = caddi(H.v[3][0], csub(g0, h0));
+}
+
+// y_new = kt H + d x + gamma y_in from the hopping sum H, complex128 (REC: gamma = -1, two
+// fused operations a part)
+template <bool REC>
+__device__ __forceinline__ void ti_combine_hop(const VecCoef<double, 1>& cf, double Vs, const Blk<double, 1>& xc,
+                                               const Blk<double, 1>& H, const Blk<double, 1>* yi,
+                                               Blk<double, 1>& yn) {
+  const double dp = fma(cf.alpha[0], Vs, cf.am[0] - cf.ab[0]), dm = fma(cf.alpha[0], Vs, -cf.am[0] - cf.ab[0]);
 #pragma unroll
-  for (int v = 0; v < VPT; ++v) {
-    cd h0 = cadd(zm.v[0][v], zm.v[1][v]), h1 = cadd(zm.v[2][v], zm.v[3][v]);
-    cd g0 = csub(zp.v[0][v], zp.v[1][v]), g1 = csub(zp.v[2][v], zp.v[3][v]);
-    cd t0 = cadd(h0, g0), t1 = csub(g0, h0), t2 = cadd(h1, g1), t3 = csub(g1, h1);
-    h0 = cadd(xm.v[0][v], xm.v[3][v]);
-    h1 = csub(xm.v[2][v], xm.v[1][v]);
-    g0 = csub(xp.v[0][v], xp.v[3][v]);
-    g1 = cadd(xp.v[2][v], xp.v[1][v]);
-    t0 = cadd(t0, cadd(h0, g0));
-    t1 = cadd(t1, csub(h1, g1));
-    t2 = cadd(t2, cadd(h1, g1));
-    t3 = cadd(t3, csub(g0, h0));
-    h0 = subi(ym.v[0][v], ym.v[3][v]);
-    h1 = subi(ym.v[2][v], ym.v[1][v]);
-    g0 = addi(yp.v[0][v], yp.v[3][v]);
-    g1 = addi(yp.v[2][v], yp.v[1][v]);
-    H.v[0][v] = cadd(t0, cadd(h0, g0));
-    H.v[1][v] = addi(t1, csub(g1, h1));
-    H.v[2][v] = cadd(t2, cadd(h1, g1));
-    H.v[3][v] = addi(t3, csub(g0, h0));
+  for (int o = 0; o < 4; ++o) {
+    const double dd = (o & 1) ? dm : dp;
+    const cplx<double> x = xc.v[o][0];
+    cplx<double> t;
+    if (yi == nullptr) {
+      t = {dd * x.re, dd * x.im};
+    } else if (REC) {
+      t = {fma(dd, x.re, -yi->v[o][0].re), fma(dd, x.im, -yi->v[o][0].im)};
+    } else {
+      t = {fma(cf.gamma[0], yi->v[o][0].re, dd * x.re), fma(cf.gamma[0], yi->v[o][0].im, dd * x.im)};
+    }
+    yn.v[o][0] = {fma(cf.kt[0], H.v[o][0].re, t.re), fma(cf.kt[0], H.v[o][0].im, t.im)};
   }
 }
 
 // y_new of one TI site from the blocks around it (Delta terms aside).  complex64 folds S and
 // D (ti_axes, ti_combine_core).  complex128 is bound by the fp64 pipe of this part (1/64 of
 // the fp32 rate: two lanes per SM), so it takes the projected hopping sum and the shortest
-// update: with gamma = -1 (every recurrence sweep after the first) y_new = kt T + (d x - y_in)
-// in two fused operations a part.  100 fp64 operations per site and vector with two dot
-// products, from 133; the KPM sweep of a 128x128x64 lattice at R = 8 takes 2.22 ms, from 2.43
-// (the z-march's eight warps do not keep the pipe busy all the time: about 75 % of its rate).
-template <typename T, int VPT>
+// update.  100 fp64 operations per site and vector with two dot
+// products, from 133 with S and D.
+template <bool REC, typename T, int VPT>
 __device__ __forceinline__ void ti_update(const VecCoef<T, VPT>& cf, T Vs, const Blk<T, VPT>& zm,
                                           const Blk<T, VPT>& xc, const Blk<T, VPT>& zp, const Blk<T, VPT>& xm,
                                           const Blk<T, VPT>& xp, const Blk<T, VPT>& ym, const Blk<T, VPT>& yp,
                                           const Blk<T, VPT>* yi, Blk<T, VPT>& yn) {
   if constexpr (sizeof(T) == 8) {
-    Blk<T, VPT> H;
-    ti_hop(zm, zp, xm, xp, ym, yp, H);
-#pragma unroll
-    for (int v = 0; v < VPT; ++v) {
-      const T dp = fma(cf.alpha[v], Vs, cf.am[v] - cf.ab[v]), dm = fma(cf.alpha[v], Vs, -cf.am[v] - cf.ab[v]);
-      const bool minus = cf.gamma[v] == T(-1);
-#pragma unroll
-      for (int o = 0; o < 4; ++o) {
-        const T dd = (o & 1) ? dm : dp;
-        const cplx<T> x = xc.v[o][v];
-        cplx<T> t;
-        if (yi == nullptr) {
-          t = {dd * x.re, dd * x.im};
-        } else if (minus) {
-          t = {fma(dd, x.re, -yi->v[o][v].re), fma(dd, x.im, -yi->v[o][v].im)};
-        } else {
-          t = {fma(cf.gamma[v], yi->v[o][v].re, dd * x.re), fma(cf.gamma[v], yi->v[o][v].im, dd * x.im)};
-        }
-        yn.v[o][v] = {fma(cf.kt[v], H.v[o][v].re, t.re), fma(cf.kt[v], H.v[o][v].im, t.im)};
-      }
-    }
+    Blk<double, 1> H;
+    hop_z_init(zm, zp, H);
+    hop_x_add(xm, xp, H);
+    hop_y_add(ym, yp, H);
+    ti_combine_hop<REC>(cf, Vs, xc, H, yi, yn);
   } else {
     Blk<T, VPT> S, D;
     ti_axes(zm, zp, xm, xp, ym, yp, S, D);
@@ -999,18 +1014,18 @@ __global__ void __launch_bounds__(256, (VPT == 1 && sizeof(T) == 4) ? 2 : 1) ti_
                                const Blk<T, VPT>& xp, const Blk<T, VPT>& ax, const Blk<T, VPT>& bx,
                                const Blk<T, VPT>& ay, const Blk<T, VPT>& by, const Blk<T, VPT>* yi,
                                Blk<T, VPT>& yn) {
-                             ti_update(cf, Vs, xm, xc, xp, ax, bx, ay, by, yi, yn);
+                             ti_update<is_recurrence(FEAT)>(cf, Vs, xm, xc, xp, ax, bx, ay, by, yi, yn);
                              if (p.g.has_delta) ti_add_delta(p.g, cf, xc, yn);
                            },
                            [&](int64_t s, const Blk<T, VPT>& xc, Blk<T, VPT>& yn) {
                              const int64_t sites[4] = {s, s, s, s};
                              epilogue<T, VPT, FEAT>(p, s, rc, xc, yn, dacc, sites);
                            });
-    if constexpr (has_dots(FEAT)) dacc.flush();  // one fp64 add per column segment
+    if constexpr (has_dots(FEAT)) dacc.flush(num_dots(FEAT));  // one fp64 add per column segment
   }
   if constexpr (has_dots(FEAT)) {
-    dacc.flush();
-    reduce_dots<VPT>(p, dacc.d);
+    dacc.flush(num_dots(FEAT));
+    reduce_dots<VPT, kMaxThreads / 32, num_dots(FEAT)>(p, dacc.d);
   }
 }
 
@@ -1067,18 +1082,18 @@ __global__ void __launch_bounds__(256) ti_sweep_xmarch(const __grid_constant__ S
       if (lym >= 0) load_at<T, VPT, true>(at(lym + x), R, ya); else zero_blk(ya);
       if (lyp >= 0) load_at<T, VPT, true>(at(lyp + x), R, yb); else zero_blk(yb);
       const T Vs = site_potential_t<T>(g, s);
-      ti_update(cf, Vs, za, xc, zb, xm, xp, ya, yb, Yin != nullptr ? &yi : nullptr, yn);
+      ti_update<is_recurrence(FEAT)>(cf, Vs, za, xc, zb, xm, xp, ya, yb, Yin != nullptr ? &yi : nullptr, yn);
       if (g.has_delta) ti_add_delta(g, cf, xc, yn);
       const int64_t sites[4] = {s, s, s, s};
       epilogue<T, VPT, FEAT>(p, s, rc, xc, yn, dacc, sites, yi);
       xm = xc;
       xc = xp;
     }
-    if constexpr (has_dots(FEAT)) dacc.flush();
+    if constexpr (has_dots(FEAT)) dacc.flush(num_dots(FEAT));
   }
   if constexpr (has_dots(FEAT)) {
-    dacc.flush();
-    reduce_dots<VPT>(p, dacc.d);
+    dacc.flush(num_dots(FEAT));
+    reduce_dots<VPT, kMaxThreads / 32, num_dots(FEAT)>(p, dacc.d);
   }
 }
 
@@ -1167,8 +1182,8 @@ __global__ void __launch_bounds__(256, 2) ti_sweep_flat(const __grid_constant__ 
     epilogue<T, VPT, FEAT>(p, s, rc, xc, yn, dacc, sites, yi);
   }
   if constexpr (has_dots(FEAT)) {
-    dacc.flush();
-    reduce_dots<VPT>(p, dacc.d);
+    dacc.flush(num_dots(FEAT));
+    reduce_dots<VPT, kMaxThreads / 32, num_dots(FEAT)>(p, dacc.d);
   }
 }
 
@@ -1278,8 +1293,8 @@ __global__ void __launch_bounds__(256) gr_sweep(const __grid_constant__ Sweep p)
     epilogue<T, VPT, FEAT>(p, c, rc, xc, yn, dacc, sites);
   }
   if constexpr (has_dots(FEAT)) {
-    dacc.flush();
-    reduce_dots<VPT>(p, dacc.d);
+    dacc.flush(num_dots(FEAT));
+    reduce_dots<VPT, kMaxThreads / 32, num_dots(FEAT)>(p, dacc.d);
   }
 }
 
@@ -1398,8 +1413,8 @@ __global__ void __launch_bounds__(256, 2) wsm_sweep(const __grid_constant__ Swee
     epilogue<T, VPT, FEAT>(p, c, rc, xc, yn, dacc, sites, yi);
   }
   if constexpr (has_dots(FEAT)) {
-    dacc.flush();
-    reduce_dots<VPT>(p, dacc.d);
+    dacc.flush(num_dots(FEAT));
+    reduce_dots<VPT, kMaxThreads / 32, num_dots(FEAT)>(p, dacc.d);
   }
 }
 
@@ -1441,11 +1456,11 @@ __global__ void __launch_bounds__(256) wsm_march_sweep(const __grid_constant__ S
           const int64_t sites[4] = {2 * c, 2 * c, 2 * c + 1, 2 * c + 1};
           epilogue<T, VPT, FEAT>(p, c, rc, xc, yn, dacc, sites);
         });
-    if constexpr (has_dots(FEAT)) dacc.flush();
+    if constexpr (has_dots(FEAT)) dacc.flush(num_dots(FEAT));
   }
   if constexpr (has_dots(FEAT)) {
-    dacc.flush();
-    reduce_dots<VPT>(p, dacc.d);
+    dacc.flush(num_dots(FEAT));
+    reduce_dots<VPT, kMaxThreads / 32, num_dots(FEAT)>(p, dacc.d);
   }
 }
 

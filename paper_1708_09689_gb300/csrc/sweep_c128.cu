@@ -27,11 +27,15 @@ static void* kernel_c128() {
 
 template <int MODEL>
 static void* pick_c128(int feat) {
+  // the flat and cp.async TI sweeps, which only a tuning entry selects, have no recurrence forms
+  constexpr bool plain = MODEL == kModelTIFlat || MODEL == kModelTIAsync || MODEL == kModelTIAsyncDeep;
   switch (feat) {
     case 0: return kernel_c128<MODEL, 0>();
     case F_DOTS: return kernel_c128<MODEL, F_DOTS>();
     case F_Z: return kernel_c128<MODEL, F_Z>();
     case F_DOTS | F_Z: return kernel_c128<MODEL, F_DOTS | F_Z>();
+    case F_KPM: return kernel_c128<MODEL, plain ? F_DOTS : F_KPM>();
+    case F_REC: return kernel_c128<MODEL, plain ? 0 : F_REC>();
     case F_ACC: return kernel_c128<MODEL, F_ACC>();
     case F_ADJ: return kernel_c128<MODEL, F_ADJ>();
     default: return nullptr;
@@ -94,7 +98,9 @@ int occupancy_c128(int model, int feat, int threads, int* blocks) {
 // ---------------------------------------------------------------- shared-memory staged TI sweep
 static void* pick_bulk_c128(int feat) {
   switch (feat) {
+    case F_REC:
     case 0: return reinterpret_cast<void*>(&ti_sweep_bulk<double, 0>);
+    case F_KPM:
     case F_DOTS: return reinterpret_cast<void*>(&ti_sweep_bulk<double, F_DOTS>);
     case F_Z: return reinterpret_cast<void*>(&ti_sweep_bulk<double, F_Z>);
     case F_DOTS | F_Z: return reinterpret_cast<void*>(&ti_sweep_bulk<double, F_DOTS | F_Z>);

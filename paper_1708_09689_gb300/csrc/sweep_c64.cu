@@ -23,6 +23,12 @@ static void* kernel_c64() {
   else return reinterpret_cast<void*>(&gr_sweep<float, VPT, FEAT>);
 }
 
+// The sweeps the library runs by itself have a KPM instantiation; the shapes only a tuning
+// entry selects (flat and cp.async TI sweeps) take the run-time dot flags.
+constexpr int kpm_feature(int model) {
+  return model == kModelTIFlat || model == kModelTIAsync || model == kModelTIAsyncDeep ? F_DOTS : F_KPM;
+}
+
 template <int MODEL, int VPT>
 static void* pick_c64(int feat) {
   switch (feat) {
@@ -30,6 +36,8 @@ static void* pick_c64(int feat) {
     case F_DOTS: return kernel_c64<MODEL, VPT, F_DOTS>();
     case F_Z: return kernel_c64<MODEL, VPT, F_Z>();
     case F_DOTS | F_Z: return kernel_c64<MODEL, VPT, F_DOTS | F_Z>();
+    case F_KPM: return kernel_c64<MODEL, VPT, kpm_feature(MODEL)>();
+    case F_REC: return kernel_c64<MODEL, VPT, 0>();  // the same arithmetic in fp32
     case F_ACC: return kernel_c64<MODEL, VPT, F_ACC>();
     default: return nullptr;
   }
@@ -78,7 +86,9 @@ int occupancy_c64(int model, int vpt, int feat, int threads, int* blocks) {
 // ---------------------------------------------------------------- shared-memory staged TI sweep
 static void* pick_bulk_c64(int feat) {
   switch (feat) {
+    case F_REC:
     case 0: return reinterpret_cast<void*>(&ti_sweep_bulk<float, 0>);
+    case F_KPM:
     case F_DOTS: return reinterpret_cast<void*>(&ti_sweep_bulk<float, F_DOTS>);
     case F_Z: return reinterpret_cast<void*>(&ti_sweep_bulk<float, F_Z>);
     case F_DOTS | F_Z: return reinterpret_cast<void*>(&ti_sweep_bulk<float, F_DOTS | F_Z>);

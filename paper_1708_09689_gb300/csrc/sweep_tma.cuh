@@ -527,7 +527,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
       return;
     }
 #pragma unroll
-    for (int d = 0; d < kNumDots; ++d)
+    for (int d = 0; d < num_dots(FEAT); ++d)
 #pragma unroll
       for (int v = 0; v < VP; ++v) {
         double t = widen(dacc.s[d][v]) + widen(dacc.c[d][v]);
@@ -860,15 +860,19 @@ static void* tma_kernel(int feat) {
     return feat == F_DOTS ? reinterpret_cast<void*>(&ti_sweep_tma<R, DEEP, NW, F_DOTS, MODEL, SL>) : nullptr;
   } else if constexpr (XM) {  // the KPM, series and plain sweeps
     switch (feat) {
+      case F_REC:
       case 0: return reinterpret_cast<void*>(&ti_sweep_tma<R, DEEP, NW, 0, MODEL, SL, true>);
       case F_DOTS: return reinterpret_cast<void*>(&ti_sweep_tma<R, DEEP, NW, F_DOTS, MODEL, SL, true>);
+      case F_KPM: return reinterpret_cast<void*>(&ti_sweep_tma<R, DEEP, NW, F_KPM, MODEL, SL, true>);
       case F_ACC: return reinterpret_cast<void*>(&ti_sweep_tma<R, DEEP, NW, F_ACC, MODEL, SL, true>);
       default: return nullptr;
     }
   } else {
     switch (feat) {
+      case F_REC:  // the same arithmetic in fp32
       case 0: return reinterpret_cast<void*>(&ti_sweep_tma<R, DEEP, NW, 0, MODEL, SL>);
       case F_DOTS: return reinterpret_cast<void*>(&ti_sweep_tma<R, DEEP, NW, F_DOTS, MODEL, SL>);
+      case F_KPM: return reinterpret_cast<void*>(&ti_sweep_tma<R, DEEP, NW, F_KPM, MODEL, SL>);
       case F_Z: return reinterpret_cast<void*>(&ti_sweep_tma<R, DEEP, NW, F_Z, MODEL, SL>);
       case F_DOTS | F_Z: return reinterpret_cast<void*>(&ti_sweep_tma<R, DEEP, NW, F_DOTS | F_Z, MODEL, SL>);
       case F_ACC: return reinterpret_cast<void*>(&ti_sweep_tma<R, DEEP, NW, F_ACC, MODEL, SL>);

@@ -30,7 +30,7 @@ int launch_tma_xm(const pvsc_lattice* lat, int feat, Sweep& p, const LaunchShape
   }
 }
 
-bool tma_xm_feature(int feat) { return feat == 0 || feat == F_DOTS || feat == F_ACC; }
+bool tma_xm_feature(int feat) { return (feat & F_Z) == 0; }
 
 int tma_error_xm(int clear, int* flag) {
   int h = 0;
