@@ -256,8 +256,16 @@ struct Sweep {
   double gscale;
   // dot products
   int dot_flags;         // bit0 xx, bit1 xy, bit2 yy
+  int dot_slices;        // rows of `partials` per slice of vectors (0, 1: every row holds every vector)
   int dot_mode;          // 0 write dots[4][R]; 1 KPM first step; 2 KPM step k; 3 KPM steps k, k+1
-  double* partials;      // [gridDim][4][R]
+  double* partials;      // [gridDim][row_len]: a row per block, dot d of vector r at d R + r
+  int row_len;           // 4 R; in a chain of KPM sweeps 2 R (two dots)
+  int grid_rows;         // set at launch: the rows this sweep writes
+  // a chain of KPM sweeps (kpm_chain): this sweep leaves its rows to the next one (defer), and sums the
+  // prev_rows rows that the one before left (step prev_k; prev_slices as dot_slices)
+  int defer;
+  int prev_rows, prev_slices, prev_k;
+  const double* prev_partials;
   unsigned* counter;     // zero before the first sweep; reset by the last block
   double* dots;          // [4][R]
   double* mu;            // [R][M]
@@ -288,43 +296,110 @@ enum AccMode { ACC_NONE = 0, ACC_INIT = 1, ACC_ADD = 2, ACC_FINAL = 4, ACC_X = 8
 // result is bitwise reproducible for a given launch configuration.
 constexpr int kMaxThreads = 256;
 
+// Output of dot d of vector r, whose sum is s (base: mu_0 or mu_1 of the doubling identities).
+__device__ __forceinline__ void write_dot(const Sweep& p, int mode, int k, int d, int r, double s, double base) {
+  double* mu = p.mu + (size_t)r * p.M;
+  if (mode == 0) {
+    p.dots[d * p.R + r] = s;
+  } else if (mode == 1) {  // KPM step 0: mu_0 = <w0|w0>, mu_1 = Re<w1|w0>
+    if (d < p.M) mu[d] = s;
+  } else {  // KPM step k: mu_2k = 2<wk|wk> - mu_0, mu_2k+1 = 2 Re<wk+1|wk> - mu_1; steps k and k+1 in one
+            // sweep (mode 3): <wk|wk>, Re<wk+1|wk>, <wk+1|wk+1>, Re<wk+2|wk+1> give mu_2k .. mu_2k+3
+    const int m = 2 * k + d;
+    if (m < p.M) mu[m] = 2.0 * s - base;
+  }
+}
+
+// Sum of column q over the rows b0, b0 + step, ... of a warp: lanes over rows, then the xor tree.
+__device__ __forceinline__ double warp_sum_rows(const double* col, int b0, int step, int nb, int row_len) {
+  double s = 0.0;
+  for (int b = b0 + step * (int)(threadIdx.x & 31); b < nb; b += 32 * step) s += __ldcg(col + (size_t)b * row_len);
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  return s;
+}
+
+// The rows that the previous sweep of a KPM chain left: every block takes one value (or, with
+// fewer blocks than values, one per warp) with one warp, beside the block's own first loads.
+// The fence, the counter and the last block's sum (round trips to L2 and a dozen dependent fp64
+// additions) are then off the end of every sweep but the last.  KPM sweeps: Weyl 256x32x32, R = 16
+// (flat) 53.5 -> 44.3 us; 256x64x8, R = 32 (z-march) 116 -> 103 us; 16^3, R = 1, complex128 15.8
+// -> 12.8 us; 256x256x64, R = 8 (kernel 7) 497 -> 488 us.
+__device__ __forceinline__ void finish_prev(const Sweep& p) {
+  if (p.prev_rows == 0) return;
+  const int nwarps = blockDim.x >> 5, warp = nwarps - 1 - (int)(threadIdx.x >> 5);  // the last warp first
+  const int SL = p.prev_slices > 1 ? p.prev_slices : 1;
+  for (int q = blockIdx.x + warp * gridDim.x; q < 2 * p.R; q += nwarps * gridDim.x) {
+    const int d = q / p.R, r = q & (p.R - 1);
+    const double base = (p.prev_k > 0 && d < p.M) ? __ldcg(p.mu + (size_t)r * p.M + d) : 0.0;
+    const double s = warp_sum_rows(p.prev_partials + q, SL > 1 ? r / (p.R / SL) : 0, SL, p.prev_rows, 2 * p.R);
+    if ((threadIdx.x & 31) == 0) write_dot(p, p.prev_k > 0 ? 2 : 1, p.prev_k, d, r, s, base);
+  }
+}
+
 // After every block has written its row of `partials`: the last block to
-// arrive sums the rows in block order and writes the outputs of dot_mode.
-__device__ __forceinline__ void finish_dots(const Sweep& p) {
+// arrive sums the rows and writes the outputs of dot_mode (a sweep that defers
+// leaves its rows to finish_prev).  Few values: a warp per value.  More than two
+// values a warp: the whole block takes part, thread t summing value q = t mod nq
+// over every (blockDim / nq)-th row (neighbouring threads on neighbouring
+// values, the loads independent of one another), then the groups as a tree, so
+// that it is about one round trip to L2 whatever R (at R = 32 on a 32x32x32
+// lattice 11 us less than a warp per value).  scratch: shared memory of blockDim
+// doubles that no thread of the block uses any more.  A KPM step reads the
+// first two dots only; with dot_slices > 1 the rows of slice s are those of
+// the blocks b with b mod dot_slices = s.
+__device__ __forceinline__ void finish_dots(const Sweep& p, double* scratch) {
+  if (p.defer) return;
   __shared__ int s_last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nwarps = blockDim.x >> 5;
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) s_last = (atomicAdd(p.counter, 1u) == gridDim.x - 1);
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  const int nb = gridDim.x;
-  for (int q = warp; q < kNumDots * p.R; q += nwarps) {
-    const int d = q / p.R, r = q % p.R;
-    if (!((p.dot_flags >> (d == 0 ? 0 : (d == 3 ? 2 : 1))) & 1)) continue;
-    if ((p.dot_mode == 1 || p.dot_mode == 2) && d > 1) continue;  // a KPM step reads the first two
-    double s = 0.0;
-    for (int b = lane; b < nb; b += 32) s += __ldcg(p.partials + (size_t)b * kNumDots * p.R + q);
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0) {
-      double* mu = p.mu + (size_t)r * p.M;
-      if (p.dot_mode == 0) {
-        p.dots[q] = s;
-      } else if (p.dot_mode == 1) {  // KPM step 0: mu_0 = <w0|w0>, mu_1 = Re<w1|w0>
-        if (d == 0) mu[0] = s;
-        if (d == 1 && p.M > 1) mu[1] = s;
-      } else if (p.dot_mode == 2) {  // KPM step k: mu_2k = 2<wk|wk> - mu_0, mu_2k+1 = 2 Re<wk+1|wk> - mu_1
-        const int k = p.kpm_k;
-        if (d == 0 && 2 * k < p.M) mu[2 * k] = 2.0 * s - __ldcg(mu);
-        if (d == 1 && 2 * k + 1 < p.M) mu[2 * k + 1] = 2.0 * s - __ldcg(mu + 1);
-      } else {  // KPM steps k and k+1 in one sweep: dots <wk|wk>, Re<wk+1|wk>,
-                // <wk+1|wk+1>, Re<wk+2|wk+1> give mu_2k .. mu_2k+3
-        const int m = 2 * p.kpm_k + d;
-        if (m < p.M) mu[m] = 2.0 * s - __ldcg(mu + (d & 1));
+  const int R = p.R, nb = gridDim.x, nthr = blockDim.x, t = threadIdx.x;
+  const bool kpm = p.dot_mode == 1 || p.dot_mode == 2;
+  const int nq = (kpm ? 2 : kNumDots) * R;  // a power of two
+  const int SL = p.dot_slices > 1 ? p.dot_slices : 1;
+  auto wanted = [&](int d) { return ((p.dot_flags >> (d == 0 ? 0 : (d == 3 ? 2 : 1))) & 1) != 0; };
+  // mu_0 or mu_1, loaded beside the rows
+  auto base_of = [&](int d, int r) {
+    return p.dot_mode >= 2 && (d & 1) < p.M ? __ldcg(p.mu + (size_t)r * p.M + (d & 1)) : 0.0;
+  };
+  if (nq <= 2 * (nthr >> 5)) {
+    for (int q = t >> 5; q < nq; q += nthr >> 5) {
+      const int d = q / R, r = q & (R - 1);
+      if (!wanted(d)) continue;
+      const double base = base_of(d, r);
+      const double s = warp_sum_rows(p.partials + q, SL > 1 ? r / (R / SL) : 0, SL, nb, p.row_len);
+      if ((t & 31) == 0) write_dot(p, p.dot_mode, p.kpm_k, d, r, s, base);
+    }
+  } else {
+    const int ng = nthr < nq ? 1 : 1 << (31 - __clz(nthr / nq));  // groups, a power of two
+    for (int q0 = 0; q0 < nq; q0 += nthr) {
+      const int q = ng > 1 ? (t & (nq - 1)) : q0 + t, grp = ng > 1 ? t / nq : 0;
+      const int d = q / R, r = q & (R - 1);
+      const bool on = q < nq && grp < ng && wanted(d);
+      double s = 0.0, base = 0.0;
+      if (on) {
+        if (grp == 0) base = base_of(d, r);
+        const double* col = p.partials + q;
+#pragma unroll 8
+        for (int b = (SL > 1 ? r / (R / SL) : 0) + SL * grp; b < nb; b += SL * ng)
+          s += __ldcg(col + (size_t)b * p.row_len);
       }
+      if (ng > 1) {
+        scratch[t] = s;
+        __syncthreads();
+        for (int half = ng >> 1; half > 0; half >>= 1) {
+          if (on && grp < half) {
+            s += scratch[t + half * nq];
+            scratch[t] = s;
+          }
+          __syncthreads();
+        }
+      }
+      if (on && grp == 0) write_dot(p, p.dot_mode, p.kpm_k, d, r, s, base);
     }
   }
   if (threadIdx.x == 0) *p.counter = 0u;
@@ -347,19 +422,19 @@ __device__ void reduce_dots(const Sweep& p, double (&acc)[kNumDots][VPT]) {
       if (lane < C) sm[warp][d][v][lane] = s;
     }
   __syncthreads();
-  double* row = p.partials + (size_t)blockIdx.x * kNumDots * p.R;
-  for (int t = threadIdx.x; t < C; t += blockDim.x) {
+  double* row = p.partials + (size_t)blockIdx.x * p.row_len;
+  for (int i = threadIdx.x; i < ND * VPT * C; i += blockDim.x) {
+    const int t = i % C, v = (i / C) % VPT, d = i / (C * VPT);
     const int stride = C < 32 ? 1 : C / 32;  // warps that carry chunk t
     const int w0 = C < 32 ? 0 : t / 32;
     const int l = C < 32 ? t : t % 32;
-    for (int d = 0; d < ND; ++d)
-      for (int v = 0; v < VPT; ++v) {
-        double s = 0.0;
-        for (int w = w0; w < nwarps; w += stride) s += sm[w][d][v][l];
-        row[d * p.R + t * VPT + v] = s;
-      }
+    if (d * p.R >= p.row_len) continue;  // a KPM sweep run with the run-time dot flags
+    double s = 0.0;
+    for (int w = w0; w < nwarps; w += stride) s += sm[w][d][v][l];
+    row[d * p.R + t * VPT + v] = s;
   }
-  finish_dots(p);
+  static_assert(MAXW * ND * VPT >= MAXW, "scratch of one double per thread");
+  finish_dots(p, &sm[0][0][0][0]);
 }
 
 

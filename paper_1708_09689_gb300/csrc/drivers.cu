@@ -88,6 +88,7 @@ static int launch_sweep_staged(const pvsc_lattice* lat, int prec, int feat, Swee
   p.zslab = (int)zs;
   const int64_t units = ntiles * ((Lz + zs - 1) / zs);
   const int grid = (int)(units < grid_max ? units : grid_max);
+  p.grid_rows = grid;
   return launch_sweep_bulk(prec, feat, grid, threads, smem, p, st);
 }
 
@@ -97,8 +98,25 @@ void sweep_init(Sweep& p, const pvsc_lattice* lat, int R, int prec) {
   p.qds = lat->qds;
   p.R = R;
   p.C = R / vpt_for(R, prec);
+  p.row_len = kNumDots * R;
   for (int r = 0; r < R; ++r) p.coef[0][r] = 1.0;
   p.cx_re = 0; p.ph_re = 1.0;
+}
+
+// A row of a KPM sweep holds two dots where a work buffer has room for four: two buffers of rows.
+void kpm_chain(const pvsc_lattice* lat, Sweep& p, double* partials, int k, bool last) {
+  p.row_len = 2 * p.R;
+  p.partials = partials + (size_t)(k & 1) * lat->sm_count * kMaxGridPerSM * p.row_len;
+  p.kpm_k = k;
+  p.dot_mode = k == 0 ? 1 : 2;
+  p.defer = last ? 0 : 1;
+}
+
+void kpm_launched(Sweep& p) {
+  p.prev_rows = p.defer ? p.grid_rows : 0;
+  p.prev_slices = p.dot_slices;
+  p.prev_k = p.kpm_k;
+  p.prev_partials = p.partials;
 }
 
 static int coef_kind(double re, double im) {
@@ -124,6 +142,7 @@ int launch_sweep_shape(const pvsc_lattice* lat, int prec, int feat, Sweep& p, La
       p.fc[t][q][0] = (float)cv[t][q];
       p.fc[t][q][1] = (float)(cv[t][q] - (double)p.fc[t][q][0]);
     }
+  p.dot_slices = 0;  // set by the sliced TMA-staged sweeps only (p may come from another launch)
   if (sh.kernel == kKernelKpm2) sh = LaunchShape{};  // a KPM-only choice: single sweeps take the default
   if (lat->g.zhalo) {  // a slab with halo planes: the z-march over its inner planes
     const int zs = sh.zslab;
@@ -219,6 +238,7 @@ int launch_sweep_shape(const pvsc_lattice* lat, int prec, int feat, Sweep& p, La
     units = (ncell * p.C + threads - 1) / threads;
   }
   const int grid = (int)(units < grid_max ? units : grid_max);
+  p.grid_rows = grid;
   return prec == PVSC_C128 ? launch_sweep_c128(model, feat, grid, threads, p, st)
                            : launch_sweep_c64(model, vpt, feat, grid, threads, p, st);
 }
@@ -449,10 +469,12 @@ int kpm_enqueue(const pvsc_lattice* lat, int R, int prec, const void* r0, uint64
   Sweep p;
   sweep_init(p, lat, R, prec);
   p.counter = reinterpret_cast<unsigned*>(work);
-  p.partials = reinterpret_cast<double*>(wptr(work, kWorkHeader));
+  double* const rows = reinterpret_cast<double*>(wptr(work, kWorkHeader));
+  p.partials = rows;
   p.mu = mu;
   p.M = M;
   p.dot_flags = 3;
+  const int nsteps = (M + 1) / 2;
   for (int r = 0; r < R; ++r) {
     p.coef[0][r] = 1.0 / a;
     p.coef[1][r] = b;
@@ -462,10 +484,11 @@ int kpm_enqueue(const pvsc_lattice* lat, int R, int prec, const void* r0, uint64
   p.yin = nullptr;
   p.yout = wb;
   p.dot_mode = 1;
+  if (!two) kpm_chain(lat, p, rows, 0, nsteps == 1);  // two steps per sweep: four dots a row, no chain
   if (int rc = launch_sweep_shape(lat, prec, F_KPM, p, sh, cs)) return rc;
+  if (!two) kpm_launched(p);
   const void* prev = x0;
   void* cur = wb;
-  const int nsteps = (M + 1) / 2;
   for (int r = 0; r < R; ++r) {
     p.coef[0][r] = 2.0 / a;
     p.coef[2][r] = -1.0;
@@ -501,7 +524,9 @@ int kpm_enqueue(const pvsc_lattice* lat, int R, int prec, const void* r0, uint64
     p.yin = prev;
     p.yout = out;
     p.kpm_k = k;
+    if (!two) kpm_chain(lat, p, rows, k, k == nsteps - 1);
     if (int rc = launch_sweep_shape(lat, prec, F_KPM, p, sh, cs)) return rc;
+    if (!two) kpm_launched(p);
     prev = cur;
     cur = out;
   }
@@ -664,31 +689,32 @@ static int kpm_moments_fx(const pvsc_lattice* lat, int R, const void* r0, uint64
     sweep_init(p, lat, R, PVSC_C128);
     p.C = R;
     p.counter = reinterpret_cast<unsigned*>(work);
-    p.partials = reinterpret_cast<double*>(wptr(work, kWorkHeader));
+    double* const rows = reinterpret_cast<double*>(wptr(work, kWorkHeader));
     p.mu = mu;
     p.M = M;
     p.dot_flags = 3;
+    const int nsteps = (M + 1) / 2;
     p.fx_d = wptr(work, L.dfx);
     p.vscale = reinterpret_cast<const double*>(wptr(work, L.vscale));
     p.x = wa;
     p.yin = nullptr;
     p.yout = wb;
-    p.dot_mode = 1;
+    kpm_chain(lat, p, rows, 0, nsteps == 1);
     p.fx_dshift = 0;
     p.fx_kt = std::llrint(std::ldexp(-0.5 * lat->g.t / a, 60));
     if (int rc = launch_sweep_fx(lat, p, sh, tuned, cs)) return rc;
+    kpm_launched(p);
     void* prev = wa;
     void* cur = wb;
     p.fx_dshift = 1;
     p.fx_kt = std::llrint(std::ldexp(-lat->g.t / a, 60));
-    p.dot_mode = 2;
-    const int nsteps = (M + 1) / 2;
     for (int k = 1; k < nsteps; ++k) {
       p.x = cur;
       p.yin = prev;
       p.yout = prev;  // w_{k+1} overwrites w_{k-1} element by element
-      p.kpm_k = k;
+      kpm_chain(lat, p, rows, k, k == nsteps - 1);
       if (int rc = launch_sweep_fx(lat, p, sh, tuned, cs)) return rc;
+      kpm_launched(p);
       std::swap(prev, cur);
     }
     return PVSC_OK;
@@ -760,9 +786,9 @@ int pvsc_kpm_sweeps(const pvsc_lattice* lat, int R, int prec, int k_begin, int k
     p.x = wk;
     p.yin = k == 0 ? nullptr : other;
     p.yout = other;
-    p.dot_mode = k == 0 ? 1 : 2;
-    p.kpm_k = k;
+    kpm_chain(lat, p, reinterpret_cast<double*>(wptr(work, kWorkHeader)), k, k == k_end - 1);
     if (int rc = launch_sweep(lat, prec, F_KPM, p, st)) return rc;
+    kpm_launched(p);
   }
   return PVSC_OK;
 }

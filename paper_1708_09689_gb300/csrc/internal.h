@@ -172,6 +172,12 @@ void sweep_init(Sweep& p, const pvsc_lattice* lat, int R, int prec);
 // p.counter inside a work buffer of at least dots_work_bytes(lat, R) bytes.
 int launch_sweep(const pvsc_lattice* lat, int prec, int feat, Sweep& p, cudaStream_t st);
 int launch_sweep_shape(const pvsc_lattice* lat, int prec, int feat, Sweep& p, LaunchShape sh, cudaStream_t st);
+// Link sweep k of a chain of KPM sweeps (consecutive k, the same Sweep p, `partials` the rows of a
+// work buffer) to the one before: each sweep but the last leaves the rows of its dot products,
+// in one of two buffers in turn, to the next one.  Call kpm_chain before the launch of a sweep and
+// kpm_launched after it.
+void kpm_chain(const pvsc_lattice* lat, Sweep& p, double* partials, int k, bool last);
+void kpm_launched(Sweep& p);
 int kpm_enqueue(const pvsc_lattice* lat, int R, int prec, const void* r0, uint64_t seed, int M, double a,
                 double b, double* mu, void* work, const LaunchShape* force, cudaStream_t cs);
 size_t dots_work_bytes(const pvsc_lattice* lat, int R);

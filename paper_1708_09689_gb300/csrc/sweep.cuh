@@ -978,6 +978,7 @@ __global__ void __launch_bounds__(256, (VPT == 1 && sizeof(T) == 4) ? 2 : 1) ti_
   const T* __restrict__ Yin = static_cast<const T*>(p.yin);
   DotAcc<T, VPT> dacc;
   dacc.init();
+  if constexpr (has_dots(FEAT)) finish_prev(p);
 
   // column groups: runs of blockDim / C consecutive columns, or with
   // p.tile_x > 0 tiles of tile_x x tile_y columns (in-plane y neighbours then
@@ -1048,6 +1049,7 @@ __global__ void __launch_bounds__(256) ti_sweep_xmarch(const __grid_constant__ S
   const T* __restrict__ Yin = static_cast<const T*>(p.yin);
   DotAcc<T, VPT> dacc;
   dacc.init();
+  if constexpr (has_dots(FEAT)) finish_prev(p);
   const int64_t nlines = Ly * Lz, nthr_lines = nlines * C;
   const int64_t nbx = (nthr_lines + blockDim.x - 1) / blockDim.x;
   const int64_t xs = p.zslab, nxs = (Lx + xs - 1) / xs;
@@ -1113,6 +1115,7 @@ __global__ void __launch_bounds__(256, 2) ti_sweep_flat(const __grid_constant__ 
   const T* __restrict__ Yin = static_cast<const T*>(p.yin);
   DotAcc<T, VPT> dacc;
   dacc.init();
+  if constexpr (has_dots(FEAT)) finish_prev(p);
   const int64_t nthr = p.g.n_sites * C;
   for (int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; tid < nthr;
        tid += (int64_t)gridDim.x * blockDim.x) {
@@ -1208,6 +1211,7 @@ __global__ void __launch_bounds__(256) gr_sweep(const __grid_constant__ Sweep p)
   const T tt = T(p.g.t);
   DotAcc<T, VPT> dacc;
   dacc.init();
+  if constexpr (has_dots(FEAT)) finish_prev(p);
   // Grid-stride loop over cells with (x, y) carried along: C is a power of
   // two and divides blockDim, so a thread keeps its chunk rc and the only
   // 64-bit divisions are the two below, once per thread.
@@ -1372,6 +1376,7 @@ __global__ void __launch_bounds__(256, 2) wsm_sweep(const __grid_constant__ Swee
   const T* __restrict__ X = static_cast<const T*>(p.x);
   DotAcc<T, VPT> dacc;
   dacc.init();
+  if constexpr (has_dots(FEAT)) finish_prev(p);
   const int cshift = __ffs(C) - 1;  // C = R / VPT is a power of two
   const int64_t cstride = ((int64_t)gridDim.x * blockDim.x) >> cshift;
   const int64_t szs = cstride / plane, rem = cstride - szs * plane;
@@ -1433,6 +1438,7 @@ __global__ void __launch_bounds__(256) wsm_march_sweep(const __grid_constant__ S
   const T* __restrict__ Yin = static_cast<const T*>(p.yin);
   DotAcc<T, VPT> dacc;
   dacc.init();
+  if constexpr (has_dots(FEAT)) finish_prev(p);
   const int64_t ncolthr = plane * C;
   const int64_t nbx = (ncolthr + blockDim.x - 1) / blockDim.x;
   const int zs = p.zslab;

@@ -114,6 +114,7 @@ __global__ void __launch_bounds__(256) ti_sweep_bulk(const __grid_constant__ Swe
   const VecCoef<T, 1> cf = load_coef<T, 1>(p, r);
   DotAcc<T, 1> dacc;
   dacc.init();
+  if constexpr (has_dots(FEAT)) finish_prev(p);
 
   const int64_t ntx = (Lx + TX - 1) / TX, nty = (Ly + TY - 1) / TY;
   const int zs = p.zslab;

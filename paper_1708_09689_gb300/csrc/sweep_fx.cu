@@ -49,6 +49,7 @@ __global__ void __launch_bounds__(256) ti_sweep_fx(const __grid_constant__ Sweep
   double dd[kNumDots][1];
 #pragma unroll
   for (int k = 0; k < kNumDots; ++k) dd[k][0] = 0.0;
+  finish_prev(p);
 
   const int64_t ncolthr = plane * C;
   const int64_t nbx = (ncolthr + blockDim.x - 1) / blockDim.x;
@@ -248,6 +249,7 @@ int launch_sweep_fx(const pvsc_lattice* lat, Sweep& p, const LaunchShape& sh, bo
   p.zslab = (int)zs;
   const int64_t units = nbx * ((Lz + zs - 1) / zs);
   const int grid = (int)(units < grid_max ? units : grid_max);
+  p.grid_rows = grid;
   void* args[] = {&p};
   PVSC_CUDA_TRY(cudaLaunchKernel(fn, dim3(grid), dim3(threads), args, smem, st));
   return PVSC_OK;

@@ -338,50 +338,42 @@ __global__ void __launch_bounds__(32 * NW, 1)
   // fastest, so the grid works on adjacent tiles at one depth); the planes of the
   // units left after the last full wave, taken in wave order, are split evenly
   // over the G blocks, a block's share being pieces of one to three units.
-  const int64_t ntiles = (int64_t)m.ntx * m.nty;
-  const int nfull = (int)(m.nunits / G);
-  const int64_t tail0 = (int64_t)nfull * G;  // first unit of the tail
-  auto unit = [&](int64_t u, uint32_t& xy, uint32_t& z0, uint32_t& n) {
-    const int64_t ch = u / ntiles, t = u - ch * ntiles, ty = t / m.ntx;
-    xy = (uint32_t)((t - ty * m.ntx) * TX) | ((uint32_t)(ty * TY) << 16);
-    z0 = (uint32_t)(ch * Lz / m.nch);
-    n = (uint32_t)((ch + 1) * Lz / m.nch) - z0;
+  const uint32_t ntiles = (uint32_t)m.ntx * (uint32_t)m.nty, nch = (uint32_t)m.nch;
+  const uint32_t nunits = (uint32_t)m.nunits;  // at most kTmaMaxUnits a block
+  const int nfull = (int)(nunits / (uint32_t)G);
+  const uint32_t tail0 = (uint32_t)nfull * (uint32_t)G;  // first unit of the tail
+  auto z_of = [&](uint32_t ch) { return ch * (uint32_t)Lz / nch; };  // first plane of a chunk (< 2^32: 16-bit factors)
+  auto xy_of = [&](uint32_t t) {
+    const uint32_t ty = t / (uint32_t)m.ntx;
+    return ((t - ty * (uint32_t)m.ntx) * TX) | ((ty * TY) << 16);
   };
   uint2* tab = reinterpret_cast<uint2*>(base + L::TAB_OFF);
   for (int i = threadIdx.x; i < nfull; i += blockDim.x) {
-    uint32_t xy, z0, n;
-    unit(vb + (int64_t)i * G, xy, z0, n);
-    tab[i] = make_uint2(xy, z0 | (n << 16));
+    const uint32_t u = (uint32_t)vb + (uint32_t)i * (uint32_t)G, ch = u / ntiles, z0 = z_of(ch);
+    tab[i] = make_uint2(xy_of(u - ch * ntiles), z0 | ((z_of(ch + 1) - z0) << 16));
   }
   __shared__ int s_ntail;
-  if (threadIdx.x == 0) {
-    // the tail spans few chunks (units are chunk-major) and a chunk's units all
-    // have its depth, so the walk goes chunk by chunk
+  if (threadIdx.x == 32 * (NW - 1)) {
+    // the planes of all units in wave order are numbered chunk by chunk, unit (ch, t) starting
+    // at ntiles z_of(ch) + t n: this block's share [lo, hi) of the tail's numbers is cut at the
+    // units it meets, each found by division (a walk over the chunks took up to 10 us of the
+    // launch on small lattices, which have a tail of many shallow chunks)
     int nt = 0;
-    if (tail0 < m.nunits) {
-      const int64_t cha = tail0 / ntiles, chb = (m.nunits - 1) / ntiles;
-      int64_t P = 0;  // planes of the tail
-      for (int64_t ch = cha; ch <= chb; ++ch) {
-        const int64_t ua = tail0 > ch * ntiles ? tail0 : ch * ntiles;
-        const int64_t ub = m.nunits < (ch + 1) * ntiles ? m.nunits : (ch + 1) * ntiles;
-        P += (ub - ua) * ((ch + 1) * Lz / m.nch - ch * Lz / m.nch);
-      }
-      const int64_t lo = P * vb / G, hi = P * (vb + 1) / G;  // this block's planes of the tail
-      int64_t off = 0;
-      for (int64_t ch = cha; ch <= chb && off < hi; ++ch) {
-        const int64_t ua = tail0 > ch * ntiles ? tail0 : ch * ntiles;
-        const int64_t ub = m.nunits < (ch + 1) * ntiles ? m.nunits : (ch + 1) * ntiles;
-        const int64_t z0 = ch * Lz / m.nch, n = (ch + 1) * Lz / m.nch - z0;  // n >= 1
-        for (int64_t k = lo > off ? (lo - off) / n : 0; ua + k < ub && off + k * n < hi; ++k) {
-          const int64_t uo = off + k * n;
-          const int64_t a = lo > uo ? lo : uo, b = hi < uo + n ? hi : uo + n;
-          if (a < b) {
-            uint32_t xy, zu, nu;
-            unit(ua + k, xy, zu, nu);
-            tab[nfull + nt++] = make_uint2(xy, (zu + (uint32_t)(a - uo)) | ((uint32_t)(b - a) << 16));
-          }
-        }
-        off += (ub - ua) * n;
+    if (tail0 < nunits) {
+      const uint32_t ct = tail0 / ntiles, zt = z_of(ct);
+      const int64_t t0 = (int64_t)ntiles * zt + (int64_t)(tail0 - ct * ntiles) * (z_of(ct + 1) - zt);
+      const uint32_t P = (uint32_t)((int64_t)ntiles * Lz - t0);  // planes of the tail (< G units of 16-bit depth)
+      int64_t p = t0 + udiv64((int64_t)P * vb, G);
+      const int64_t hi = t0 + udiv64((int64_t)P * (vb + 1), G);
+      while (p < hi) {
+        const uint32_t zq = (uint32_t)udiv64(p, ntiles);
+        const uint32_t ch = ((zq + 1) * nch - 1) / (uint32_t)Lz;  // the last chunk with z_of(ch) <= zq
+        const uint32_t z0 = z_of(ch), n = z_of(ch + 1) - z0;
+        const int64_t q = p - (int64_t)ntiles * z0;
+        const uint32_t t = (uint32_t)udiv64(q, n), a = (uint32_t)(q - (int64_t)t * n);
+        const uint32_t len = (int64_t)(n - a) < hi - p ? n - a : (uint32_t)(hi - p);
+        tab[nfull + nt++] = make_uint2(xy_of(t), (z0 + a) | (len << 16));
+        p += len;
       }
     }
     s_ntail = nt;
@@ -490,6 +482,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
     }
   }
 
+  if constexpr (has_dots(FEAT)) finish_prev(p);  // while the first copies are in flight
   const int c = lane % L::CPS;
   const int q = lane / L::CPS;
   const int cg = c + sl * L::CPS;  // the chunk (complex64) or vector (fixed point) in the block
@@ -765,22 +758,20 @@ __global__ void __launch_bounds__(32 * NW, 1)
     // arrival counter stays consistent)
     const double* wd = reinterpret_cast<const double*>(base + L::DOT_OFF);
     constexpr int RV = FX ? R / 2 : R;  // vectors of a slice
-    constexpr int RVF = RV * SL;        // of the block (zeros outside this block's slice)
-    double* row = p.partials + (size_t)blockIdx.x * kNumDots * RVF;
-    for (int t = threadIdx.x; t < kNumDots * RVF; t += blockDim.x) {
-      const int d = t / RVF, r = t - d * RVF - sl * RV;
+    constexpr int RVF = RV * SL;        // of the block (this block writes its slice's)
+    double* row = p.partials + (size_t)blockIdx.x * p.row_len;
+    constexpr int ND = FX ? 2 : num_dots(FEAT);
+    for (int t = threadIdx.x; t < ND * RV; t += blockDim.x) {
+      const int d = t / RV, r = t - d * RV;
       double sum = 0.0;
-      if (r >= 0 && r < RV) {
-        if constexpr (FX) {
-          if (d < 2)
-            for (int w = 0; w < NCW; ++w) sum += wd[w * kNumDots * 2 * L::CPS + d * L::CPS + r];
-        } else {
-          for (int w = 0; w < NCW; ++w) sum += wd[((w * kNumDots + d) * 2 + (r & 1)) * L::CPS + (r >> 1)];
-        }
+      if constexpr (FX) {
+        for (int w = 0; w < NCW; ++w) sum += wd[w * kNumDots * 2 * L::CPS + d * L::CPS + r];
+      } else {
+        for (int w = 0; w < NCW; ++w) sum += wd[((w * kNumDots + d) * 2 + (r & 1)) * L::CPS + (r >> 1)];
       }
-      row[t] = sum;
+      row[d * RVF + sl * RV + r] = sum;
     }
-    finish_dots(p);
+    finish_dots(p, reinterpret_cast<double*>(base));  // the rings are drained
   }
 }
 
@@ -914,6 +905,7 @@ static int launch_tma_r(const pvsc_lattice* lat, int feat, Sweep& p, const Launc
   PVSC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 32 * NW, L::SMEM));
   if (occ < 1) return set_error(PVSC_ERR_CUDA, "the TMA-staged sweep does not fit an SM");
   p.C = L::CPS;
+  p.dot_slices = SL;
   p.tile_x = L::TX;
   p.tile_y = L::TY;
   TmaMaps m;
@@ -936,13 +928,13 @@ static int launch_tma_r(const pvsc_lattice* lat, int feat, Sweep& p, const Launc
   m.nch = nch;
   m.nunits = ntiles * nch;  // per slice
   p.zslab = (int)((Lz + nch - 1) / nch);
-  // no more blocks than units, unless the shape asks to spread (blocks_per_sm
-  // = 1): with fewer units than SMs, splitting the columns' planes over all SMs
-  // was measured slower on the Weyl cuboid (77.9 -> 72.2 GLUP/s: pieces at
-  // staggered depths lose the halo strips' L2 reuse) and is left to the
-  // autotuner; blocks left without a plane issue no copy
-  const bool spread = sh.blocks_per_sm == 1;
+  // with fewer units than SMs the planes are spread over every SM when the shape asks for it
+  // (blocks_per_sm = 1) or leaves the chunks to auto_chunks, whose count assumes it (64x64x64,
+  // R = 4: 29 us a KPM sweep, 158 us on one block per unit); an explicit chunk depth without it
+  // keeps one block per unit.  Blocks left without a plane issue no copy
+  const bool spread = sh.blocks_per_sm == 1 || sh.zslab <= 0;
   const int grid = (int)(SL * (m.nunits < grid_max && !spread ? m.nunits : grid_max));
+  p.grid_rows = grid;
   void* args[] = {&p, &m};
   // with programmatic dependent launch: all of a sweep's blocks are resident at
   // once (grid <= SMs x occupancy), so the next sweep's blocks, which wait for
