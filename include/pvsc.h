@@ -567,6 +567,9 @@ typedef struct {
                   /* the next sweep's blocks set up on free SMs and wait for the */
                   /* previous sweep to complete before touching global memory (same */
                   /* results; environment PVSC_NO_PDL=1 launches them plainly). */
+                  /* Without an entry, complex64 sweeps of TI and Weyl lattices that fill the */
+                  /* chip run kernel 7's tiles (any Lx), the others the z-march (TI) or a */
+                  /* flat cell sweep (Weyl); pvsc_get_tuning then still reads 256 threads, kernel 0. */
                   /* PVSC_Q64 (KPM on TI lattices) takes kernels 0, 2, 3 (threads a */
                   /* multiple of R, one vector per thread, no tile) and 7 for R = 1 .. 32 */
                   /* (any Lx): the tiles, rings and variants of the complex64 layout */

@@ -67,6 +67,26 @@ static void cache_store(const std::string& key, const pvsc_tuning& t) {
   std::fclose(f);
 }
 
+// The untuned sweep as a candidate, where no tuning entry can select it (the TMA-staged tiles of a
+// lattice with Lx no multiple of 4): threads = 0 stands for it in the list and in the cache file,
+// and installing it removes the entry.  The caller is told the defaults that pvsc_get_tuning reads.
+static bool untuned_is_its_own(const pvsc_lattice* lat, int R, int prec) {
+  return tma_sweep_default(lat, R, prec) && !tma_sweep_possible(lat, R, prec);
+}
+
+static void install(pvsc_lattice* lat, int R, int prec, const pvsc_tuning& t) {
+  if (t.threads > 0) lat->tuning[{R, prec}] = t;
+  else lat->tuning.erase({R, prec});
+}
+
+static pvsc_tuning reported(pvsc_tuning t, int R, int prec) {
+  if (t.threads == 0) {
+    t.threads = 256;
+    t.vpt = vpt_for(R, prec);
+  }
+  return t;
+}
+
 }  // namespace pvsc
 
 using namespace pvsc;
@@ -80,9 +100,9 @@ extern "C" int pvsc_autotune_op(pvsc_lattice* lat, int R, int prec, int op, pvsc
   const std::string key = cache_key(lat, R, prec, op);
   pvsc_tuning cached;
   if (cache_lookup(key, &cached)) {
-    lat->tuning[{R, prec}] = cached;
+    install(lat, R, prec, cached);
     drop_graphs(lat);
-    if (best) *best = cached;
+    if (best) *best = reported(cached, R, prec);
     return PVSC_OK;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -137,7 +157,7 @@ extern "C" int pvsc_autotune_op(pvsc_lattice* lat, int R, int prec, int op, pvsc
   // + dots), series (the accumulating sweep and the two plain ones that follow
   // it), apply (plain)
   auto time_one = [&](const pvsc_tuning& cand, float* ms) -> int {
-    lat->tuning[{R, prec}] = cand;
+    install(lat, R, prec, cand);
     Sweep p;
     sweep_init(p, lat, R, prec);
     for (int r = 0; r < R; ++r) {
@@ -187,6 +207,7 @@ extern "C" int pvsc_autotune_op(pvsc_lattice* lat, int R, int prec, int op, pvsc
   // candidate list: z-marching (all shapes), and for TI the flat, prefetching
   // and shared-memory staged sweeps in a few shapes each
   std::vector<pvsc_tuning> cands;
+  if (untuned_is_its_own(lat, R, prec)) cands.push_back(pvsc_tuning{0, 0, 0, 0.f, 0, 0, 0, 0});
   for (int vpt : vpt_c) {
     const int C = R / vpt;
     for (int th : {64, 128, 256}) {
@@ -251,10 +272,10 @@ extern "C" int pvsc_autotune_op(pvsc_lattice* lat, int R, int prec, int op, pvsc
     if (had) lat->tuning[{R, prec}] = old; else lat->tuning.erase({R, prec});
     return rc;
   }
-  lat->tuning[{R, prec}] = win;
+  install(lat, R, prec, win);
   drop_graphs(lat);
   cache_store(key, win);
-  if (best) *best = win;
+  if (best) *best = reported(win, R, prec);
   return PVSC_OK;
 }
 

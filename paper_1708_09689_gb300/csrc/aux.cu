@@ -69,10 +69,18 @@ __global__ void seed_potential_kernel(double* V, int64_t n, uint64_t key, double
     V[s] = W * (hash_uniform(key, (uint64_t)s) - 0.5);
 }
 
-__global__ void potential_f32_kernel(const double* __restrict__ V, float* __restrict__ V32, int64_t n) {
+// V32p (may be null): the same values again in rows of Lp instead of Lx
+__global__ void potential_f32_kernel(const double* __restrict__ V, float* __restrict__ V32, float* __restrict__ V32p,
+                                     int64_t Lx, int64_t Lp, int64_t n) {
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n;
-       s += (int64_t)gridDim.x * blockDim.x)
-    V32[s] = (float)V[s];
+       s += (int64_t)gridDim.x * blockDim.x) {
+    const float v = (float)V[s];
+    V32[s] = v;
+    if (V32p != nullptr) {
+      const int64_t row = udiv64(s, Lx);
+      V32p[row * Lp + (s - row * Lx)] = v;
+    }
+  }
 }
 
 __global__ void get_potential_kernel(Geometry g, double* out) {
@@ -272,8 +280,10 @@ int launch_seed_potential(double* V, int64_t n, uint64_t seed, double W, cudaStr
   return PVSC_OK;
 }
 
-int launch_potential_f32(const double* V, float* V32, int64_t n, cudaStream_t st) {
-  potential_f32_kernel<<<grid_for(n, 256), 256, 0, st>>>(V, V32, n);
+int launch_potential_f32(const pvsc_lattice* lat, cudaStream_t st) {
+  const int64_t n = lat->g.n_sites, Lx = lat->g.L[0];
+  potential_f32_kernel<<<grid_for(n, 256), 256, 0, st>>>(lat->V_dev, lat->V32_dev, lat->V32p_dev, Lx,
+                                                         padded_row(Lx), n);
   PVSC_CUDA_TRY(cudaGetLastError());
   return PVSC_OK;
 }

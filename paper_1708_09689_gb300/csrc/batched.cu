@@ -337,6 +337,7 @@ static int kpm_per_lattice(const pvsc_lattice* const* lats, int n, int R, int pr
   std::stable_sort(order.begin(), order.end(),
                    [&](int x, int y) { return lats[x]->g.n_sites > lats[y]->g.n_sites; });
   LaunchShape force;
+  force.tuned = true;
   force.kernel = kKernelTma;
   force.threads = bs.threads;
   std::vector<uint64_t> uid = {6, (uint64_t)n, (uint64_t)R, (uint64_t)prec, (uint64_t)M,

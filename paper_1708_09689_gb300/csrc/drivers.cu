@@ -20,6 +20,7 @@ static LaunchShape shape_for(const pvsc_lattice* lat, int R, int prec) {
   LaunchShape sh;
   auto it = lat->tuning.find({R, prec});
   if (it != lat->tuning.end()) {
+    sh.tuned = true;
     sh.threads = it->second.threads;
     sh.blocks_per_sm = it->second.blocks_per_sm;
     sh.zslab = it->second.zslab;
@@ -148,6 +149,12 @@ int launch_sweep_shape(const pvsc_lattice* lat, int prec, int feat, Sweep& p, La
     const int zs = sh.zslab;
     sh = LaunchShape{};
     sh.zslab = zs;
+  }
+  if (!sh.tuned && !(feat & F_ADJ) && tma_sweep_default(lat, p.R, prec)) {
+    // sixteen warps where the accumulator is read and written (its loads are the longest waits)
+    LaunchShape d;
+    d.threads = (feat & F_ACC) ? 512 : 256;
+    return launch_sweep_tma(lat, feat, p, d, st);
   }
   if (sh.kernel == kKernelTma || sh.kernel == kKernelTmaX) {
     p.tile_x = p.tile_y = 0;

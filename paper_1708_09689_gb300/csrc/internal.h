@@ -40,6 +40,7 @@ struct LaunchShape {
                           // 4 two KPM steps per sweep (tile_x x tile_y tiles),
                           // 5 z-marching over tile_x x tile_y column tiles, 6 marching along x,
                           // 7 TMA-staged plane tiles (warp-specialised)
+  bool tuned = false;     // the fields above are a tuning entry's; else the library's own choice
 };
 
 // kernel-selector "model" values of the flat and the cp.async-prefetching TI
@@ -97,7 +98,9 @@ constexpr int kKernelXMarch = 6;
 // TI (and Weyl-cell) sweep with TMA-staged z-plane tiles (sweep_tma.cu):
 // complex64, R = 4 .. 64, Lx a multiple of 4
 constexpr int kKernelTma = 7;
-bool tma_sweep_possible(const pvsc_lattice* lat, int R, int prec);
+bool tma_sweep_possible(const pvsc_lattice* lat, int R, int prec);  // what a tuning entry may select
+bool tma_sweep_fits(const pvsc_lattice* lat, int R, int prec);      // what the kernel runs: any Lx
+bool tma_sweep_default(const pvsc_lattice* lat, int R, int prec);   // the choice of an untuned sweep
 int launch_sweep_tma(const pvsc_lattice* lat, int feat, Sweep& p, const LaunchShape& sh, cudaStream_t st);
 // the same tiles marching along x (tiles over (y, z) columns): TI, complex64; the
 // fused step with z falls back to kernel 7
@@ -134,6 +137,8 @@ struct pvsc_lattice {
   pvsc::Geometry g{};
   double* V_dev = nullptr;  // owned when v_mode == 1
   float* V32_dev = nullptr; // fp32 copy of V_dev for complex64 sweeps
+  float* V32p_dev = nullptr;  // TI / Weyl, Lx no multiple of 4: V32 again in rows of padded_row(Lx), whose
+                              // 16-byte row stride the TMA-staged sweeps' copies need (null: no room)
   pvsc::QDots* qd_dev = nullptr;  // quantum-dot array parameters (v_mode 3)
   pvsc::QDScal qds{};             // and the scalars the sweeps take as parameters
   int v_source = 0;
@@ -157,6 +162,8 @@ struct pvsc_lattice {
 };
 
 namespace pvsc {
+
+inline int64_t padded_row(int64_t Lx) { return (Lx + 3) / 4 * 4; }
 
 constexpr int kMaxGridPerSM = 16;
 constexpr size_t kWorkHeader = 256;  // counters at the start of every work buffer
@@ -198,7 +205,7 @@ int launch_scale_init(const void* x128, double2* acc, double cr, double ci, int6
                       cudaStream_t st);
 int launch_seed_potential(double* V, int64_t n, uint64_t seed, double W, cudaStream_t st);
 int launch_get_potential(const Geometry& g, double* out, cudaStream_t st);
-int launch_potential_f32(const double* V, float* V32, int64_t n, cudaStream_t st);
+int launch_potential_f32(const pvsc_lattice* lat, cudaStream_t st);  // V_dev -> V32_dev (and V32p_dev)
 int launch_gershgorin(const Geometry& g, double* out, int grid, cudaStream_t st);
 int launch_neighbours(const Geometry& g, int64_t* nbr, cudaStream_t st);
 int launch_adjoint_top(const pvsc_lattice* lat, int R, const double2* G, double sr, double si,

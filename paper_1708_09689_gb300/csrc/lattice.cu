@@ -60,6 +60,17 @@ size_t dots_work_bytes(const pvsc_lattice* lat, int R) {
   return kWorkHeader + (size_t)lat->sm_count * kMaxGridPerSM * kNumDots * R * sizeof(double);
 }
 
+// The row-padded fp32 potential (see V32p_dev); without room for it the sweeps of
+// this lattice stay off the TMA-staged tiles.
+static void alloc_padded_potential(pvsc_lattice* lat) {
+  const Geometry& g = lat->g;
+  if (g.model == PVSC_GRAPHENE || g.L[0] % 4 == 0) return;
+  if (cudaMalloc(&lat->V32p_dev, sizeof(float) * (size_t)(padded_row(g.L[0]) * g.L[1] * g.L[2])) != cudaSuccess) {
+    lat->V32p_dev = nullptr;
+    cudaGetLastError();
+  }
+}
+
 }  // namespace pvsc
 
 pvsc_lattice::~pvsc_lattice() {
@@ -69,6 +80,7 @@ pvsc_lattice::~pvsc_lattice() {
   }
   if (V_dev) cudaFree(V_dev);
   if (V32_dev) cudaFree(V32_dev);
+  if (V32p_dev) cudaFree(V32p_dev);
   if (qd_dev) cudaFree(qd_dev);
 }
 
@@ -199,6 +211,7 @@ int pvsc_lattice_create(const pvsc_lattice_desc* desc, void* stream, pvsc_lattic
       delete lat;
       return set_error(PVSC_ERR_OOM, "cudaMalloc of V failed: %s", cudaGetErrorString(e));
     }
+    alloc_padded_potential(lat);
     g.V = lat->V_dev;
     g.V32 = lat->V32_dev;
     g.v_mode = 1;
@@ -209,7 +222,7 @@ int pvsc_lattice_create(const pvsc_lattice_desc* desc, void* stream, pvsc_lattic
                           desc->v_source == PVSC_V_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, st);
       if (e != cudaSuccess) rc = set_error(PVSC_ERR_CUDA, "copy of V failed: %s", cudaGetErrorString(e));
     }
-    if (rc == PVSC_OK) rc = launch_potential_f32(lat->V_dev, lat->V32_dev, g.n_sites, st);
+    if (rc == PVSC_OK) rc = launch_potential_f32(lat, st);
   } else if (desc->v_source == PVSC_V_ON_THE_FLY) {
     g.v_mode = 2;
   } else if (desc->v_source == PVSC_V_QDOT) {
@@ -260,6 +273,7 @@ int pvsc_set_potential(pvsc_lattice* lat, const double* V_dev, void* stream) {
     cudaError_t e = cudaMalloc(&lat->V_dev, sizeof(double) * lat->g.n_sites);
     if (e == cudaSuccess) e = cudaMalloc(&lat->V32_dev, sizeof(float) * lat->g.n_sites);
     if (e != cudaSuccess) return set_error(PVSC_ERR_OOM, "cudaMalloc of V failed: %s", cudaGetErrorString(e));
+    alloc_padded_potential(lat);
     lat->g.V = lat->V_dev;
     lat->g.V32 = lat->V32_dev;
     lat->g.v_mode = 1;
@@ -269,7 +283,7 @@ int pvsc_set_potential(pvsc_lattice* lat, const double* V_dev, void* stream) {
   lat->gersh_valid = false;
   PVSC_CUDA_TRY(cudaMemcpyAsync(lat->V_dev, V_dev, sizeof(double) * lat->g.n_sites,
                                 cudaMemcpyDeviceToDevice, static_cast<cudaStream_t>(stream)));
-  return launch_potential_f32(lat->V_dev, lat->V32_dev, lat->g.n_sites, static_cast<cudaStream_t>(stream));
+  return launch_potential_f32(lat, static_cast<cudaStream_t>(stream));
 }
 
 int pvsc_get_potential(const pvsc_lattice* lat, double* V_out_dev, void* stream) {

@@ -39,10 +39,11 @@ static bool tma_units_fit(const pvsc_lattice* lat, int64_t tiles_per_slice, int 
 
 // The kernel's unit table holds the (x0, y0, z0, planes) of a block's units in
 // 16-bit fields, at most kTmaMaxUnits of them (one z-chunk per column at least).
-bool tma_sweep_possible(const pvsc_lattice* lat, int R, int prec) {
+// The potential comes in 16-byte rows: a stored one with Lx no multiple of 4 in the padded copy.
+bool tma_sweep_fits(const pvsc_lattice* lat, int R, int prec) {
   const Geometry& g = lat->g;
-  if (!((g.model == PVSC_TI || g.model == PVSC_WSM) && prec == PVSC_C64 && valid_R(R) && g.L[0] % 4 == 0 &&
-        g.L[0] < 65536 && g.L[1] < 65536 && g.L[2] < 65536))
+  if (!((g.model == PVSC_TI || g.model == PVSC_WSM) && prec == PVSC_C64 && valid_R(R) && g.L[0] < 65536 &&
+        g.L[1] < 65536 && g.L[2] < 65536 && !(g.v_mode == 1 && g.L[0] % 4 != 0 && !lat->V32p_dev)))
     return false;
   const int64_t ntiles = R == 1    ? tma_tiles<1>(g)
                          : R == 2  ? tma_tiles<2>(g)
@@ -54,6 +55,10 @@ bool tma_sweep_possible(const pvsc_lattice* lat, int R, int prec) {
   return tma_units_fit(lat, ntiles, R);
 }
 
+
+bool tma_sweep_possible(const pvsc_lattice* lat, int R, int prec) {
+  return lat->g.L[0] % 4 == 0 && tma_sweep_fits(lat, R, prec);
+}
 
 static void tma_tiles_of(int R, int* tx_large, int* ty_large, int* tx_deep, int* ty_deep) {
   switch (R) {
@@ -86,10 +91,29 @@ bool tma_tile_valid(int R, int tile_x, int tile_y) {
   return (tile_x == a && tile_y == b) || (tile_x == c && tile_y == d);
 }
 
+// An untuned complex64 sweep runs the tiles where there is enough work for their fixed cost (a
+// launch of about 8 us: barriers, unit table, first copies, one 200 KB block per SM, against 5 us
+// of the register sweeps) and the large tile is at least half full.  The flat Weyl sweep, with half
+// the state of a TI thread, keeps up longer: up to 2^21 site-vectors it is left only by narrow
+// blocks (R <= 4) or for well filled tiles.  KPM sweeps, register sweep -> tiles, us: TI 16x16x16
+// R = 8: 7.9 -> 8.5, R = 32: 11.1 -> 8.5; 32x32x32 R = 1: 6.9 -> 8.1, R = 4: 12.7 -> 9.0;
+// 101x87x53 R = 4: 63.8 -> 43.7; 128x128x64 R = 8: 184 -> 142; tiles 12/32 full (12x200x100, R = 1):
+// 15.9 -> 17.3.  Weyl 32x32x32 R = 8: 10.2 -> 8.5; 40x48x20 (20/24 full) R = 16: 11.7 -> 14.7;
+// 48x48x48 R = 16: 19.6 -> 20.5, R = 4: 14.7 -> 12.4; 256x32x32 R = 16: 44.0 -> 39.5.
+bool tma_sweep_default(const pvsc_lattice* lat, int R, int prec) {
+  const int64_t work = lat->g.n_sites * R;
+  const bool wsm = lat->g.model == PVSC_WSM;
+  if (lat->g.zhalo || !tma_sweep_fits(lat, R, prec) || work <= (wsm ? 1 << 17 : 1 << 16)) return false;
+  int tx, ty, dx, dy;
+  tma_tiles_of(R, &tx, &ty, &dx, &dy);
+  const int64_t Lx = wsm ? lat->g.L[0] / 2 : lat->g.L[0], Ly = lat->g.L[1];
+  const double full = (double)(Lx * Ly) / (double)(((Lx + tx - 1) / tx * tx) * ((Ly + ty - 1) / ty * ty));
+  return full >= (wsm && R >= 8 && work <= (1 << 21) ? 0.85 : 0.5);
+}
+
 int launch_sweep_tma(const pvsc_lattice* lat, int feat, Sweep& p, const LaunchShape& sh, cudaStream_t st) {
-  if (!tma_sweep_possible(lat, p.R, PVSC_C64))
-    return set_error(PVSC_ERR_UNSUPPORTED, "the TMA-staged sweep needs a complex64 TI or Weyl lattice "
-                     "and Lx a multiple of 4");
+  if (!tma_sweep_fits(lat, p.R, PVSC_C64))
+    return set_error(PVSC_ERR_UNSUPPORTED, "the TMA-staged sweep needs a complex64 TI or Weyl lattice");
   if (p.R >= 32) return launch_tma_sliced(lat, feat, p, sh, st);
   if (p.R <= 2) return launch_tma_narrow(lat, feat, p, sh, st);
   if (lat->g.model == PVSC_WSM) return launch_tma_wide(lat, feat, p, sh, st);

@@ -833,10 +833,13 @@ static int encode_maps(const pvsc_lattice* lat, const Sweep& p, TmaMaps& m) {
     if (int rc = tile5(&m.yi, p.yin, L::TX, L::TY)) return rc;
   m.v_tma = MODEL == kModelTIFx ? 1 : (!XM && lat->g.v_mode == 1);
   if (m.v_tma) {
+    // rows of 4-byte words, in the padded copy where Lx is no multiple of 4 (16-byte strides)
+    const bool padded = MODEL != kModelTIFx && lat->g.L[0] % 4 != 0;
+    const cuuint64_t pitch = padded ? 4 * padded_row(lat->g.L[0]) : 4 * vf * Lx;
     const cuuint64_t vd[3] = {vf * Lx, Ly, Lz};  // per site
-    const cuuint64_t vs[2] = {4 * vf * Lx, 4 * vf * Lx * Ly};
+    const cuuint64_t vs[2] = {pitch, pitch * Ly};
     const cuuint32_t vb[3] = {(cuuint32_t)(vf * L::TX), (cuuint32_t)L::TY, 1};
-    void* vptr = MODEL == kModelTIFx ? const_cast<void*>(p.fx_d) : static_cast<void*>(const_cast<float*>(lat->g.V32));
+    void* vptr = MODEL == kModelTIFx ? const_cast<void*>(p.fx_d) : static_cast<void*>(padded ? lat->V32p_dev : lat->V32_dev);
     const CUresult r = enc(&m.v, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, vptr, vd, vs, vb,
                            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
