@@ -446,6 +446,13 @@ int pvsc_kpm_density(int R, int M, const double* mu, int kernel, double lambda, 
                      double scale, int NE, const double* E, double* rho, void* stream);
 
 /*
+ * pvsc_kpm_density of n spectra on the same energies in one launch: mu is
+ * device [n][R][M], rho device [n][NE]; spectrum i from the R rows mu[i].
+ */
+int pvsc_kpm_spectra(int n, int R, int M, const double* mu, int kernel, double lambda, double a, double b,
+                     double scale, int NE, const double* E, double* rho, void* stream);
+
+/*
  * The states psi(k, nu) of Eq. ak on a cubic lattice with O orbitals per site
  * (TI: O = 4, Weyl semimetal: O = 2), for nk k-points k[3 q .. 3 q + 2]
  * (HOST array of 3 nk doubles, components along x, y, z in radians per

@@ -90,6 +90,7 @@ _SIGNATURES = {
     "pvsc_cheb_step_noalloc": (_i, [_vp, _i, _i, _vp, _vp, _vp, _dp, _dp, _dp, _dp, _i, _vp, _vp]),
     "pvsc_kpm_moments": (_i, [_vp, _i, _i, _vp, _u64, _i, _d, _d, _vp, _vp, _sz, _vp]),
     "pvsc_kpm_density": (_i, [_i, _i, _vp, _i, _d, _d, _d, _d, _i, _vp, _vp, _vp]),
+    "pvsc_kpm_spectra": (_i, [_i, _i, _i, _vp, _i, _d, _d, _d, _d, _i, _vp, _vp, _vp]),
     "pvsc_chebfd": (_i, [_vp, _vp, _d, _d, _vp, _vp, _vp, _vp, _vp, _vp, _sz, _vp]),
     "pvsc_chebfd_work_bytes": (_sz, [_vp, _i, _i, _i]),
     "pvsc_bloch_vectors": (_i, [_vp, _i, ctypes.POINTER(_d), _i, _vp, _vp]),
@@ -531,9 +532,11 @@ def spectral_function(lat: Lattice, ks, M: int, a, b, E, prec: int = C64,
     k-point (one call, R = O nk), summed per k-point; returns (nk, NE) float64."""
     psi = bloch_vectors(lat, ks, prec)
     mu = kpm_moments(lat, M, a, b, r0=psi, work=work)
-    E = torch.as_tensor(E, dtype=torch.float64, device="cuda")
-    O = lat.orbitals
-    return torch.stack([kpm_density(mu[O * q:O * q + O], E, a, b, kernel, lam) for q in range(len(ks))])
+    E = torch.as_tensor(E, dtype=torch.float64, device="cuda").contiguous()
+    out = torch.empty((len(ks),) + tuple(E.shape), dtype=torch.float64, device=mu.device)
+    _check(_lib.pvsc_kpm_spectra(len(ks), lat.orbitals, int(M), _ptr(mu), int(kernel), float(lam), float(a), float(b),
+                                 1.0, E.numel(), _ptr(E), _ptr(out), _stream()))
+    return out
 
 
 class ChebFDParams(ctypes.Structure):

@@ -9,15 +9,24 @@
 
 namespace pvsc {
 
+// What every damping factor of a spectrum shares: cot(pi/(M + 1)) (Jackson) or sinh(lambda) (Lorentz).
+__device__ __forceinline__ double damping_common(int kernel, int M, double lambda) {
+  if (kernel == PVSC_KERNEL_JACKSON) {
+    const double q = M_PI / (M + 1);
+    return cos(q) / sin(q);
+  }
+  return kernel == PVSC_KERNEL_LORENTZ ? sinh(lambda) : 1.0;
+}
+
 // Damping factor g_k of M moments: 0 none, 1 Jackson, 2 Lorentz(lambda).
-__device__ __forceinline__ double damping(int kernel, int k, int M, double lambda) {
+__device__ __forceinline__ double damping(int kernel, int k, int M, double lambda, double common) {
   if (kernel == PVSC_KERNEL_JACKSON) {
     const double q = M_PI / (M + 1);
     double s, c;
     sincos(q * k, &s, &c);
-    return ((M - k + 1) * c + s * (cos(q) / sin(q))) / (M + 1);
+    return ((M - k + 1) * c + s * common) / (M + 1);
   }
-  if (kernel == PVSC_KERNEL_LORENTZ) return sinh(lambda * (1.0 - (double)k / M)) / sinh(lambda);
+  if (kernel == PVSC_KERNEL_LORENTZ) return sinh(lambda * (1.0 - (double)k / M)) / common;
   return 1.0;
 }
 
@@ -27,13 +36,22 @@ constexpr int kDensityChunk = 1024;  // series coefficients staged in shared mem
 // x_j = (E_j - b)/a, rho = 0 for |x_j| >= 1.  One thread per energy; the block
 // forms the coefficients c_k = g_k sum_r mu_k^r chunk by chunk in shared
 // memory and every thread runs the Chebyshev recurrence T_{k+1} = 2 x T_k - T_{k-1}
-// through them.
-__global__ void __launch_bounds__(256) kpm_density_kernel(int R, int M, const double* __restrict__ mu,
+// through them.  Block row y is spectrum y (mu and rho follow one another).  All
+// of it is fp64, two lanes per SM: blocks of 64 threads and all spectra of a
+// call in one launch put it on as many SMs as there are (eight spectra of 1024
+// energies, 256 moments: eight launches of four 256-thread blocks, 375 us, to
+// one of 128 blocks, 24 us).
+constexpr int kDensityThreads = 64;
+__global__ void __launch_bounds__(kDensityThreads) kpm_density_kernel(int R, int M, const double* __restrict__ mu,
                                                           int kernel, double lambda, double a, double b,
                                                           double scale, int NE,
                                                           const double* __restrict__ E,
                                                           double* __restrict__ rho) {
   __shared__ double c[kDensityChunk];
+  __shared__ double common;
+  mu += (size_t)blockIdx.y * R * M;
+  rho += (size_t)blockIdx.y * NE;
+  if (threadIdx.x == 0) common = damping_common(kernel, M, lambda);
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   const double x = j < NE ? (E[j] - b) / a : 2.0;
   const bool inside = fabs(x) < 1.0;
@@ -46,7 +64,7 @@ __global__ void __launch_bounds__(256) kpm_density_kernel(int R, int M, const do
       const int k = k0 + i;
       double s = 0.0;
       for (int r = 0; r < R; ++r) s += mu[(size_t)r * M + k];
-      c[i] = (k == 0 ? 1.0 : 2.0) * damping(kernel, k, M, lambda) * s;
+      c[i] = (k == 0 ? 1.0 : 2.0) * damping(kernel, k, M, lambda, common) * s;
     }
     __syncthreads();
     if (inside) {
@@ -70,53 +88,67 @@ struct KPoints {
   double k[16][3];
 };
 
-template <typename T>
-__global__ void bloch_kernel(const Geometry g, int O, int R, const KPoints kp, T* out) {
-  const int64_t n = O * g.n_sites * (int64_t)R;  // complex elements
+// A thread forms the phase of one (site, k-point) and writes its O x O corner of the site's
+// block (O consecutive vectors of every orbital, zeros off the diagonal): one sincos per phase,
+// every lane at work.  A thread per element left 8 of 32 lanes with a phase and ran the fp64
+// range reduction for each of them: 1505 us for eight k-points on 256x64x8 sites.
+template <typename T, int O>
+__global__ void __launch_bounds__(256) bloch_kernel(const Geometry g, int nk, const __grid_constant__ KPoints kp,
+                                                    T* out) {
+  const int64_t n = g.n_sites * nk;
   const double inv = 1.0 / sqrt((double)g.n_sites);
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = udiv64(e, R);  // site * O + orbital
-    const int r = (int)(e - i * R);
-    const int64_t s = i / O;
-    const int o = (int)(i - s * O);
-    double re = 0.0, im = 0.0;
-    if (r % O == o) {
-      const int q = r / O;
-      const int64_t yz = udiv64(s, g.L[0]);
-      const int64_t x = s - yz * g.L[0];
-      const int64_t z = udiv64(yz, g.L[1]);
-      const int64_t y = yz - z * g.L[1];
-      const double ph = kp.k[q][0] * (double)x + kp.k[q][1] * (double)y + kp.k[q][2] * (double)z;
-      double sn, cs;
-      sincos(ph, &sn, &cs);
-      re = cs * inv;
-      im = sn * inv;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t s = udiv64(e, nk);
+    const int q = (int)(e - s * nk);
+    const int64_t yz = udiv64(s, g.L[0]);
+    const int64_t x = s - yz * g.L[0];
+    const int64_t z = udiv64(yz, g.L[1]);
+    const int64_t y = yz - z * g.L[1];
+    const double ph = kp.k[q][0] * (double)x + kp.k[q][1] * (double)y + kp.k[q][2] * (double)z;
+    double sn, cs;
+    sincos(ph, &sn, &cs);
+    const T re = T(cs * inv), im = T(sn * inv);
+    T* p = out + 2 * (s * O * (int64_t)(O * nk) + O * q);
+#pragma unroll
+    for (int o = 0; o < O; ++o) {
+      if constexpr (sizeof(T) == 8) {
+        double2* d = reinterpret_cast<double2*>(p + 2 * (int64_t)o * O * nk);
+#pragma unroll
+        for (int nu = 0; nu < O; ++nu) d[nu] = nu == o ? make_double2(re, im) : make_double2(0.0, 0.0);
+      } else {
+        float4* d = reinterpret_cast<float4*>(p + 2 * (int64_t)o * O * nk);
+#pragma unroll
+        for (int nu = 0; nu < O; nu += 2)
+          d[nu / 2] = make_float4(nu == o ? re : 0.f, nu == o ? im : 0.f, nu + 1 == o ? re : 0.f, nu + 1 == o ? im : 0.f);
+      }
     }
-    out[2 * e] = T(re);
-    out[2 * e + 1] = T(im);
   }
 }
 
-static int launch_kpm_density(int R, int M, const double* mu, int kernel, double lambda, double a,
-                       double b, double scale, int NE, const double* E, double* rho,
-                       cudaStream_t st) {
-  const int threads = 256;
-  const int grid = (NE + threads - 1) / threads;
-  kpm_density_kernel<<<grid, threads, 0, st>>>(R, M, mu, kernel, lambda, a, b, scale, NE, E, rho);
+static int kpm_spectra(int n, int R, int M, const double* mu, int kernel, double lambda, double a, double b,
+                       double scale, int NE, const double* E, double* rho, cudaStream_t st) {
+  if (n < 1 || n > 65535) return set_error(PVSC_ERR_ARG, "n = %d spectra: need 1 .. 65535", n);
+  if (R < 1 || M < 1 || NE < 0) return set_error(PVSC_ERR_ARG, "need R >= 1, M >= 1, NE >= 0");
+  if (kernel != PVSC_KERNEL_NONE && kernel != PVSC_KERNEL_JACKSON && kernel != PVSC_KERNEL_LORENTZ)
+    return set_error(PVSC_ERR_ARG, "unknown damping kernel %d", kernel);
+  if (kernel == PVSC_KERNEL_LORENTZ && !(std::isfinite(lambda) && lambda > 0))
+    return set_error(PVSC_ERR_ARG, "the Lorentz kernel needs lambda > 0");
+  if (!(std::isfinite(a) && a > 0) || !std::isfinite(b) || !std::isfinite(scale))
+    return set_error(PVSC_ERR_ARG, "need a > 0 and finite b, scale");
+  if (NE == 0) return PVSC_OK;
+  if (int rc = check_ptr(mu, "mu")) return rc;
+  if (int rc = check_ptr(E, "E")) return rc;
+  if (int rc = check_ptr(rho, "rho")) return rc;
+  const dim3 grid((NE - 1) / kDensityThreads + 1, n);
+  kpm_density_kernel<<<grid, kDensityThreads, 0, st>>>(R, M, mu, kernel, lambda, a, b, scale, NE, E, rho);
   PVSC_CUDA_TRY(cudaGetLastError());
   return PVSC_OK;
 }
 
-static int launch_bloch(const Geometry& g, int O, int R, int prec, const KPoints& kp, void* out,
-                        cudaStream_t st) {
-  const int64_t n = O * g.n_sites * (int64_t)R;
-  int64_t blocks = (n + 255) / 256;
-  if (blocks > 65535) blocks = 65535;
-  if (prec == PVSC_C128)
-    bloch_kernel<double><<<(int)blocks, 256, 0, st>>>(g, O, R, kp, static_cast<double*>(out));
-  else
-    bloch_kernel<float><<<(int)blocks, 256, 0, st>>>(g, O, R, kp, static_cast<float*>(out));
+template <typename T, int O>
+static int launch_bloch(const Geometry& g, int nk, const KPoints& kp, void* out, cudaStream_t st) {
+  const int64_t blocks = (g.n_sites * nk + 255) / 256;
+  bloch_kernel<T, O><<<(int)(blocks < 65535 ? blocks : 65535), 256, 0, st>>>(g, nk, kp, static_cast<T*>(out));
   PVSC_CUDA_TRY(cudaGetLastError());
   return PVSC_OK;
 }
@@ -129,19 +161,12 @@ extern "C" {
 
 int pvsc_kpm_density(int R, int M, const double* mu, int kernel, double lambda, double a, double b,
                      double scale, int NE, const double* E, double* rho, void* stream) {
-  if (R < 1 || M < 1 || NE < 0) return set_error(PVSC_ERR_ARG, "need R >= 1, M >= 1, NE >= 0");
-  if (kernel != PVSC_KERNEL_NONE && kernel != PVSC_KERNEL_JACKSON && kernel != PVSC_KERNEL_LORENTZ)
-    return set_error(PVSC_ERR_ARG, "unknown damping kernel %d", kernel);
-  if (kernel == PVSC_KERNEL_LORENTZ && !(std::isfinite(lambda) && lambda > 0))
-    return set_error(PVSC_ERR_ARG, "the Lorentz kernel needs lambda > 0");
-  if (!(std::isfinite(a) && a > 0) || !std::isfinite(b) || !std::isfinite(scale))
-    return set_error(PVSC_ERR_ARG, "need a > 0 and finite b, scale");
-  if (NE == 0) return PVSC_OK;
-  if (int rc = check_ptr(mu, "mu")) return rc;
-  if (int rc = check_ptr(E, "E")) return rc;
-  if (int rc = check_ptr(rho, "rho")) return rc;
-  return launch_kpm_density(R, M, mu, kernel, lambda, a, b, scale, NE, E, rho,
-                            static_cast<cudaStream_t>(stream));
+  return kpm_spectra(1, R, M, mu, kernel, lambda, a, b, scale, NE, E, rho, static_cast<cudaStream_t>(stream));
+}
+
+int pvsc_kpm_spectra(int n, int R, int M, const double* mu, int kernel, double lambda, double a, double b,
+                     double scale, int NE, const double* E, double* rho, void* stream) {
+  return kpm_spectra(n, R, M, mu, kernel, lambda, a, b, scale, NE, E, rho, static_cast<cudaStream_t>(stream));
 }
 
 int pvsc_bloch_vectors(const pvsc_lattice* lat, int nk, const double* k, int prec, void* out,
@@ -160,7 +185,10 @@ int pvsc_bloch_vectors(const pvsc_lattice* lat, int nk, const double* k, int pre
   KPoints kp{};  // passed by value in the kernel parameters
   for (int q = 0; q < nk; ++q)
     for (int d = 0; d < 3; ++d) kp.k[q][d] = k[3 * q + d];
-  return launch_bloch(lat->g, O, O * nk, prec, kp, out, static_cast<cudaStream_t>(stream));
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (prec == PVSC_C128)
+    return O == 4 ? launch_bloch<double, 4>(lat->g, nk, kp, out, st) : launch_bloch<double, 2>(lat->g, nk, kp, out, st);
+  return O == 4 ? launch_bloch<float, 4>(lat->g, nk, kp, out, st) : launch_bloch<float, 2>(lat->g, nk, kp, out, st);
 }
 
 }  // extern "C"
