@@ -43,8 +43,8 @@ __global__ void scale_init_kernel(const double2* __restrict__ x, double2* __rest
   }
 }
 
-// u_M = sigma G and grad[site] += gscale Re sum conj(u_M) w (one thread per site, R = 1 block)
-__global__ void adjoint_top_kernel(const double2* __restrict__ G, double sr, double si,
+// G <- ph G, then u_M = sigma G and grad[site] += gscale Re sum conj(u_M) w (one thread per site, R = 1 block)
+__global__ void adjoint_top_kernel(double2* __restrict__ G, double pr, double pi, double sr, double si,
                                    double2* __restrict__ uM, const double2* __restrict__ w,
                                    double gscale, double* __restrict__ grad, int64_t n_sites,
                                    int per_site) {
@@ -53,7 +53,9 @@ __global__ void adjoint_top_kernel(const double2* __restrict__ G, double sr, dou
     double g = 0.0;
     for (int k = 0; k < per_site; ++k) {
       const int64_t e = s * per_site + k;
-      const double2 a = G[e];
+      const double2 h = G[e];
+      const double2 a = make_double2(pr * h.x - pi * h.y, pr * h.y + pi * h.x);
+      G[e] = a;
       const double2 u = make_double2(sr * a.x - si * a.y, sr * a.y + si * a.x);
       uM[e] = u;
       const double2 b = w[e];
@@ -264,12 +266,12 @@ int launch_scale_init(const void* x128, double2* acc, double cr, double ci, int6
   return PVSC_OK;
 }
 
-int launch_adjoint_top(const pvsc_lattice* lat, int R, const double2* G, double sr, double si,
+int launch_adjoint_top(const pvsc_lattice* lat, int R, double2* G, double pr, double pi, double sr, double si,
                        double2* uM, const double2* w, double gscale, double* grad,
                        cudaStream_t st) {
   const int per_site = orbitals_of(lat->g.model) * R;
-  adjoint_top_kernel<<<grid_for(lat->g.n_sites, 256), 256, 0, st>>>(G, sr, si, uM, w, gscale, grad,
-                                                                  lat->g.n_sites, per_site);
+  adjoint_top_kernel<<<grid_for(lat->g.n_sites, 256), 256, 0, st>>>(G, pr, pi, sr, si, uM, w, gscale,
+                                                                  grad, lat->g.n_sites, per_site);
   PVSC_CUDA_TRY(cudaGetLastError());
   return PVSC_OK;
 }

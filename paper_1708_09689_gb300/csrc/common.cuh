@@ -239,10 +239,16 @@ struct Sweep {
   void* yout2;           // two-step KPM sweep: w_{k+2} (yout holds w_{k+1})
   void* z;               // may be null
   double coef[4][kMaxR]; // alpha, beta, gamma, delta per vector
+  // set at launch from coef (set_products): alpha beta, alpha m and the hopping weight (TI -alpha t / 2,
+  // graphene -alpha t) of complex128 sweeps; these three, alpha, gamma and delta in fp32 of complex64 ones
+  union {
+    double pd[3][kMaxR];
+    float pf[6][kMaxR];
+  };
   // series accumulation (complex128 accumulator)
   int acc_mode;          // AccMode bits (below)
   int acc_kind;          // set at launch: bits 0-1 kind of cx, 2-3 of cy, 4-5 of cz (0 general, 1 real,
-                         // 2 imaginary, 3 zero or no such term)
+                         // 2 imaginary, 3 zero or no such term), ACC_SIGMA_IM: sigma imaginary (else real)
   double2* acc;
   double2* acc_out;      // final: written here
   double cx_re, cx_im, cy_re, cy_im, ph_re, ph_im;
@@ -286,6 +292,7 @@ struct Sweep {
 // its value before the sweep (the series writes y_new over it); FINAL writes
 // ph acc_new to acc_out instead of acc.  YIN comes with X, and with neither
 // INIT nor XSRC.
+constexpr int ACC_SIGMA_IM = 64;  // a bit of acc_kind
 enum AccMode { ACC_NONE = 0, ACC_INIT = 1, ACC_ADD = 2, ACC_FINAL = 4, ACC_X = 8, ACC_XSRC = 16, ACC_YIN = 32 };
 
 // ---------------------------------------------------------------- deterministic dot reduction

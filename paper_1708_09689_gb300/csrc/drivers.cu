@@ -120,6 +120,28 @@ void kpm_launched(Sweep& p) {
   p.prev_partials = p.partials;
 }
 
+// The products of the coefficients that the sweeps use, in their arithmetic type (in a thread they
+// are fp64 multiplications and conversions, which the compiler may repeat for every site, and a
+// thread of a small complex128 sweep updates one or two cells).
+void set_products(const pvsc_lattice* lat, int prec, Sweep& p) {
+  const double hop = lat->g.model == PVSC_GRAPHENE ? -1.0 : -0.5;
+  for (int r = 0; r < p.R; ++r) {
+    const double a = p.coef[0][r], ab = a * p.coef[1][r], am = a * lat->g.m, kt = hop * a * lat->g.t;
+    if (prec == PVSC_C128) {
+      p.pd[0][r] = ab;
+      p.pd[1][r] = am;
+      p.pd[2][r] = kt;
+    } else {
+      p.pf[0][r] = (float)ab;
+      p.pf[1][r] = (float)am;
+      p.pf[2][r] = (float)kt;
+      p.pf[3][r] = (float)a;
+      p.pf[4][r] = (float)p.coef[2][r];
+      p.pf[5][r] = (float)p.coef[3][r];
+    }
+  }
+}
+
 static int coef_kind(double re, double im) {
   return (im == 0.0 ? 1 : 0) | (re == 0.0 ? 2 : 0);  // 1 real, 2 imaginary, 3 zero, 0 general
 }
@@ -136,7 +158,9 @@ int launch_sweep_shape(const pvsc_lattice* lat, int prec, int feat, Sweep& p, La
                                    "and no INIT or XSRC");
   // an absent x or y_in term has the kind of a zero weight (3)
   p.acc_kind = ((p.acc_mode & ACC_X) ? coef_kind(p.cx_re, p.cx_im) : 3) | (coef_kind(p.cy_re, p.cy_im) << 2) |
-               (((p.acc_mode & ACC_YIN) ? coef_kind(p.cz_re, p.cz_im) : 3) << 4);
+               (((p.acc_mode & ACC_YIN) ? coef_kind(p.cz_re, p.cz_im) : 3) << 4) |
+               ((feat & F_ADJ) && p.sg_re == 0.0 ? ACC_SIGMA_IM : 0);
+  set_products(lat, prec, p);
   const double cv[3][2] = {{p.cx_re, p.cx_im}, {p.cy_re, p.cy_im}, {p.cz_re, p.cz_im}};
   for (int t = 0; t < 3; ++t)
     for (int q = 0; q < 2; ++q) {
@@ -189,6 +213,7 @@ int launch_sweep_shape(const pvsc_lattice* lat, int prec, int feat, Sweep& p, La
   const bool wsm = lat->g.model == PVSC_WSM;
   const bool wsm_flat = wsm && (lat->tuning.count({p.R, prec}) == 0 || sh.kernel == 1);
   const bool qd = lat->g.model == PVSC_GRAPHENE && lat->g.v_mode == 3;
+  const bool by_site = lat->g.model == PVSC_GRAPHENE && !qd && prec == PVSC_C128 && gr_by_site(feat);
   const bool xmarch = lat->g.model == PVSC_TI && sh.kernel == kKernelXMarch;
   const int model = xmarch ? kModelTIXMarch
                     : flat ? kModelTIFlat
@@ -243,8 +268,12 @@ int launch_sweep_shape(const pvsc_lattice* lat, int prec, int feat, Sweep& p, La
     // graphene: 4-site cells; Weyl semimetal: cells of two sites
     const int64_t ncell = lat->g.model == PVSC_WSM ? lat->g.n_sites / 2 : lat->g.L[0] * lat->g.L[1];
     units = (ncell * p.C + threads - 1) / threads;
+    if (by_site) units = (lat->g.n_sites * p.R + threads - 1) / threads;
   }
-  const int grid = (int)(units < grid_max ? units : grid_max);
+
+  // no rows of dot products: blocks beyond the resident ones even out the SMs' shares
+  const int64_t grid_cap = by_site ? 8 * grid_max : grid_max;
+  const int grid = (int)(units < grid_cap ? units : grid_cap);
   p.grid_rows = grid;
   return prec == PVSC_C128 ? launch_sweep_c128(model, feat, grid, threads, p, st)
                            : launch_sweep_c64(model, vpt, feat, grid, threads, p, st);
@@ -897,11 +926,13 @@ int pvsc_cheb_adjoint_step(const pvsc_lattice* lat, int R, int prec, const void*
   auto Wk = [&](int k) -> void* { return k == 0 ? const_cast<void*>(psi_s) : wptr(work, kWorkHeader + (k - 1) * vb); };
   void* ubuf[2] = {wptr(work, kWorkHeader + (size_t)(M > 1 ? M - 1 : 0) * vb),
                    wptr(work, kWorkHeader + (size_t)(M > 1 ? M : 1) * vb)};
-  const cd cphi = std::exp(cd(0, b * dt));  // conj(e^{-i b dt})
-  auto sigma = [&](int k) { return std::conj(cw[k]) * cphi; };
+  // the weights sigma_k = conj(cw_k) cphi share the phase cphi = conj(e^{-i b dt}): G is multiplied
+  // by it once, and what is left is real (k even) or imaginary (k odd)
+  const cd cphi = std::exp(cd(0, b * dt));
+  auto sigma = [&](int k) { return std::conj(cw[k]); };
   const int64_t n = lat->g.n_sites * orbitals_of(lat->g.model);
   if (M == 0) {
-    const cd s0 = sigma(0);
+    const cd s0 = sigma(0) * cphi;
     return launch_scale_init(G, static_cast<double2*>(G), s0.real(), s0.imag(), n, st);
   }
   Sweep p;
@@ -916,11 +947,11 @@ int pvsc_cheb_adjoint_step(const pvsc_lattice* lat, int R, int prec, const void*
     p.yout = Wk(k);
     if (int rc = launch_sweep(lat, prec, F_REC, p, st)) return rc;
   }
-  // u_M = sigma_M G, grad += (f_{M-1}/a) Re conj(u_M) w_{M-1}
+  // G <- cphi G, u_M = sigma_M G, grad += (f_{M-1}/a) Re conj(u_M) w_{M-1}
   {
     const cd s = sigma(M);
     const double f = (M - 1 == 0) ? 1.0 : 2.0;
-    if (int rc = launch_adjoint_top(lat, R, static_cast<const double2*>(G), s.real(), s.imag(),
+    if (int rc = launch_adjoint_top(lat, R, static_cast<double2*>(G), cphi.real(), cphi.imag(), s.real(), s.imag(),
                                     static_cast<double2*>(ubuf[0]), static_cast<const double2*>(Wk(M - 1)),
                                     f / a, dLdV, st))
       return rc;

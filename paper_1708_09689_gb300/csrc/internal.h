@@ -185,6 +185,7 @@ int launch_sweep_shape(const pvsc_lattice* lat, int prec, int feat, Sweep& p, La
 // kpm_launched after it.
 void kpm_chain(const pvsc_lattice* lat, Sweep& p, double* partials, int k, bool last);
 void kpm_launched(Sweep& p);
+void set_products(const pvsc_lattice* lat, int prec, Sweep& p);  // Sweep::pd or pf from coef
 int kpm_enqueue(const pvsc_lattice* lat, int R, int prec, const void* r0, uint64_t seed, int M, double a,
                 double b, double* mu, void* work, const LaunchShape* force, cudaStream_t cs);
 size_t dots_work_bytes(const pvsc_lattice* lat, int R);
@@ -208,7 +209,7 @@ int launch_get_potential(const Geometry& g, double* out, cudaStream_t st);
 int launch_potential_f32(const pvsc_lattice* lat, cudaStream_t st);  // V_dev -> V32_dev (and V32p_dev)
 int launch_gershgorin(const Geometry& g, double* out, int grid, cudaStream_t st);
 int launch_neighbours(const Geometry& g, int64_t* nbr, cudaStream_t st);
-int launch_adjoint_top(const pvsc_lattice* lat, int R, const double2* G, double sr, double si,
+int launch_adjoint_top(const pvsc_lattice* lat, int R, double2* G, double pr, double pi, double sr, double si,
                        double2* uM, const double2* w, double gscale, double* grad,
                        cudaStream_t st);
 

@@ -22,6 +22,7 @@ static void* kernel_c128() {
   else if constexpr (MODEL == kModelWSMMarch) return reinterpret_cast<void*>(&wsm_march_sweep<double, 1, FEAT>);
   else if constexpr (MODEL == kModelGrapheneQD) return reinterpret_cast<void*>(&gr_sweep<double, 1, FEAT, true>);
   else if constexpr (MODEL == kModelTIXMarch) return reinterpret_cast<void*>(&ti_sweep_xmarch<double, 1, FEAT>);
+  else if constexpr (gr_by_site(FEAT)) return reinterpret_cast<void*>(&gr_site_sweep<FEAT>);
   else return reinterpret_cast<void*>(&gr_sweep<double, 1, FEAT>);
 }
 

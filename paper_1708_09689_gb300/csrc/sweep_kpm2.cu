@@ -300,6 +300,7 @@ int kpm2_check_tile(int TX, int TY, int R) {
 int launch_kpm2_sweep(const pvsc_lattice* lat, Sweep& p, const LaunchShape& sh, cudaStream_t st) {
   if (p.R < 2 || p.R % 2) return set_error(PVSC_ERR_ARG, "two-step KPM sweep needs R >= 2");
   p.dot_slices = 0;
+  set_products(lat, PVSC_C64, p);
   p.C = p.R / 2;
   int TX = 0, TY = 0;
   kpm2_default_tile(p.C, TX, TY);

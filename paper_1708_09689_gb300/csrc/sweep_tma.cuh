@@ -487,7 +487,10 @@ __global__ void __launch_bounds__(32 * NW, 1)
   const int q = lane / L::CPS;
   const int cg = c + sl * L::CPS;  // the chunk (complex64) or vector (fixed point) in the block
   VecCoef<float, VP> cf;
-  if constexpr (!FX) cf = load_coef<float, VP>(p, cg);
+  if constexpr (!FX) {
+    cf = load_coef<float, VP>(p, cg);
+    hold_coef(cf);
+  }
   DotAcc<float, VP> dacc;  // compensated fp32 sums; their fp64 part lives in shared memory
   dacc.init();
   // fixed point: exact per-unit dot sums of this thread's vector c, the
