@@ -410,7 +410,10 @@ size_t pvsc_propagate_adjoint_work_bytes(const pvsc_lattice* lat, int R, int eve
  * phase counter, bounded spin waits), so the lattices advance independently.
  * Launch shape (threads per block, z-slab planes, blocks per SM): the tuning
  * entry (R, prec) of lats[0] if one is set, else 256 threads, whole columns
- * (one unit per column and step) and the occupancy maximum.  An entry with
+ * (one unit per column and step) and the occupancy maximum.  Without an entry
+ * a complex64 batch of large lattices (2^18 site-vectors on average) runs as
+ * the chains below, on the sweeps an untuned lattice takes, if work holds them
+ * (pvsc_batched_work_bytes does).  An entry with
  * kernel 7 (complex64, every lattice eligible for kernel 7) runs each
  * lattice's KPM instead as its own chain of TMA-staged sweeps (threads 256 or
  * 512: the large tile on 8 or 16 warps), the chains on a few streams forked

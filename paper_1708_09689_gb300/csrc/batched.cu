@@ -269,6 +269,7 @@ static size_t batch_header_bytes(int n) {
 struct BatchShape {
   int threads = 256, zs = 0, bps = 0;
   bool per_lattice = false;  // kernel 7: every lattice's KPM on the TMA-staged sweep
+  bool tuned = false;
 };
 static BatchShape batch_shape(const pvsc_lattice* l0, int R, int prec) {
   BatchShape sh;
@@ -276,6 +277,7 @@ static BatchShape batch_shape(const pvsc_lattice* l0, int R, int prec) {
   auto it = l0->tuning.find({R, prec});
   if (it != l0->tuning.end()) {
     const pvsc_tuning& t = it->second;
+    sh.tuned = true;
     if (t.threads >= 32 && t.threads <= kMaxThreads && t.threads % 32 == 0 && t.threads % C == 0)
       sh.threads = t.threads;
     if (t.zslab > 0) sh.zs = t.zslab;
@@ -308,15 +310,33 @@ static size_t per_lattice_bytes(const pvsc_lattice* lat, int R, int prec) {
   return ((dots_work_bytes(lat, R) + 255) & ~size_t(255)) + 2 * vec_bytes(lat, R, prec);
 }
 
+static size_t chains_bytes(const pvsc_lattice* const* lats, int n, int R, int prec) {
+  size_t total = 0;
+  for (int i = 0; i < n; ++i) total += (per_lattice_bytes(lats[i], R, prec) + 255) & ~size_t(255);
+  return total;
+}
+
+// Without a tuning entry on the first lattice a complex64 batch runs as chains of untuned sweeps
+// where its lattices hold 2^18 site-vectors on average.  The persistent launch -> chains, 64 moments:
+// sixteen cubes of 24 .. 64, R = 16: 22.7 -> 13.5 ms, R = 4 (413 k site-vectors): 8.1 -> 4.8 ms (6.5
+// with the graph's capture in a first call, 8.3 persistent); of 16 .. 28, R = 16 (176 k): 3.1 -> 2.3 ms,
+// but 3.9 against 3.2 in a first call.
+static bool chains_default(const pvsc_lattice* const* lats, int n, int R, int prec, const BatchShape& sh) {
+  if (sh.tuned || prec != PVSC_C64) return false;
+  int64_t work = 0;
+  for (int i = 0; i < n; ++i) {
+    if (!lats[i] || lats[i]->g.model != PVSC_TI || lats[i]->g.zhalo || !tma_sweep_fits(lats[i], R, prec)) return false;
+    work += lats[i]->g.n_sites * R;
+  }
+  return work >= (int64_t)n << 18;
+}
+
 static int kpm_per_lattice(const pvsc_lattice* const* lats, int n, int R, int prec, const uint64_t* seeds, int M,
                            const double* a, const double* b, double* mu, void* work, size_t work_bytes,
                            const BatchShape& bs, cudaStream_t st) {
   std::vector<size_t> off(n);
-  size_t total = 0;
-  for (int i = 0; i < n; ++i) {
-    off[i] = total;
-    total += (per_lattice_bytes(lats[i], R, prec) + 255) & ~size_t(255);
-  }
+  const size_t total = chains_bytes(lats, n, R, prec);
+  for (int i = 1; i < n; ++i) off[i] = off[i - 1] + ((per_lattice_bytes(lats[i - 1], R, prec) + 255) & ~size_t(255));
   if (work_bytes < total) return set_error(PVSC_ERR_ARG, "work buffer too small: %zu < %zu", work_bytes, total);
   static std::mutex mu_streams;
   static cudaStream_t pool[kBatchStreams];
@@ -336,12 +356,25 @@ static int kpm_per_lattice(const pvsc_lattice* const* lats, int n, int R, int pr
   for (int i = 0; i < n; ++i) order[i] = i;
   std::stable_sort(order.begin(), order.end(),
                    [&](int x, int y) { return lats[x]->g.n_sites > lats[y]->g.n_sites; });
-  LaunchShape force;
-  force.tuned = true;
-  force.kernel = kKernelTma;
+  // Sweeps of several chains share the chip: a lattice that is less than half of the batch runs one
+  // block per unit, in units deep enough for the batch to fill the SMs twice over (spread over every
+  // SM as a sweep on its own is, the chains would run one after another: sixteen cubes of 20^3, R = 16,
+  // 8.3 us a sweep and cube)
+  const double sms = (double)lats[0]->sm_count;
+  double planes = 0.0;  // tile planes of one sweep of every lattice
+  std::vector<double> lat_planes(n);
+  for (int i = 0; i < n; ++i) {
+    lat_planes[i] = (double)tma_large_tiles(lats[i], R) * lats[i]->g.L[2];
+    planes += lat_planes[i];
+  }
+  const double depth = 0.5 * planes / sms;
+  LaunchShape force;  // untuned: every sweep the library's own choice
+  force.tuned = bs.tuned;
+  force.kernel = bs.tuned ? kKernelTma : 0;
   force.threads = bs.threads;
   std::vector<uint64_t> uid = {6, (uint64_t)n, (uint64_t)R, (uint64_t)prec, (uint64_t)M,
-                               (uint64_t)(uintptr_t)mu, (uint64_t)(uintptr_t)work, (uint64_t)bs.threads};
+                               (uint64_t)(uintptr_t)mu, (uint64_t)(uintptr_t)work, (uint64_t)bs.threads,
+                               (uint64_t)bs.tuned};
   for (int i = 0; i < n; ++i) {
     uint64_t ab[2];
     std::memcpy(&ab[0], &a[i], 8);
@@ -357,8 +390,13 @@ static int kpm_per_lattice(const pvsc_lattice* const* lats, int n, int R, int pr
       for (int j = 1; j < kBatchStreams; ++j)
         if (load[j] < load[k]) k = j;
       load[k] += (double)lats[i]->g.n_sites;
+      LaunchShape sh = force;
+      if (lat_planes[i] < 0.5 * planes) {
+        sh.side_by_side = true;
+        sh.zslab = (int)std::min<double>(std::max(depth, 1.0), (double)lats[i]->g.L[2]);
+      }
       if (int rc = kpm_enqueue(lats[i], R, prec, nullptr, seeds[i], M, a[i], b[i], mu + (size_t)i * R * M,
-                               static_cast<char*>(work) + off[i], &force, pool[k]))
+                               static_cast<char*>(work) + off[i], &sh, pool[k]))
         return rc;
     }
     for (int k = 0; k < kBatchStreams; ++k) {
@@ -423,12 +461,10 @@ size_t pvsc_batched_work_bytes(const pvsc_lattice* const* lats, int n, int R, in
   size_t total = 0;
   if (!lats[0]) return 0;
   const BatchShape sh = batch_shape(lats[0], R, prec);
-  if (sh.per_lattice && per_lattice_possible(lats, n, R, prec)) {
-    for (int i = 0; i < n; ++i) total += (per_lattice_bytes(lats[i], R, prec) + 255) & ~size_t(255);
-    return total;
-  }
+  if (sh.per_lattice && per_lattice_possible(lats, n, R, prec)) return chains_bytes(lats, n, R, prec);
   if (batched_layout(lats, n, R, prec, M, L, &total, sh.threads, sh.zs) != PVSC_OK) return 0;
-  return total;
+  // either form of an untuned batch may run in it
+  return chains_default(lats, n, R, prec, sh) ? std::max(total, chains_bytes(lats, n, R, prec)) : total;
 }
 
 int pvsc_kpm_moments_batched(const pvsc_lattice* const* lats, int n, int R, int prec,
@@ -452,6 +488,11 @@ int pvsc_kpm_moments_batched(const pvsc_lattice* const* lats, int n, int R, int 
     return kpm_per_lattice(lats, n, R, prec, seeds, M, a, b, mu, work, work_bytes, sh,
                            static_cast<cudaStream_t>(stream));
   }
+  // (an injected stall is one of the persistent launch's waits; a work buffer that holds only
+  // the persistent launch gets it)
+  if (!g_inject_stall && chains_default(lats, n, R, prec, sh) && work_bytes >= chains_bytes(lats, n, R, prec))
+    return kpm_per_lattice(lats, n, R, prec, seeds, M, a, b, mu, work, work_bytes, sh,
+                           static_cast<cudaStream_t>(stream));
   const int threads = sh.threads;
   std::vector<BatchLat> L;
   size_t total = 0;
@@ -559,8 +600,15 @@ int pvsc_autotune_batched(pvsc_lattice* const* lats, int n, int R, int prec, con
   const bool had = saved != l0->tuning.end();
   const pvsc_tuning old = had ? saved->second : pvsc_tuning{};
   size_t wmax = 0;
+  // the untuned batch, where its chains are no entry's (some Lx no multiple of 4): threads = 0
+  auto install = [&](const pvsc_tuning& t) {
+    if (t.threads > 0) l0->tuning[{R, prec}] = t; else l0->tuning.erase({R, prec});
+  };
+  l0->tuning.erase({R, prec});
+  if (!per_lattice_possible(lats, n, R, prec) && chains_default(lats, n, R, prec, batch_shape(l0, R, prec)))
+    cands.push_back(pvsc_tuning{0, 0, 0, 0.f, 0, 0, 0, 0});
   for (const pvsc_tuning& c : cands) {
-    l0->tuning[{R, prec}] = c;
+    install(c);
     wmax = std::max(wmax, pvsc_batched_work_bytes(lats, n, R, prec, M));
   }
   void *work = nullptr, *mu = nullptr;
@@ -582,7 +630,7 @@ int pvsc_autotune_batched(pvsc_lattice* const* lats, int n, int R, int prec, con
   cudaEventCreate(&e1);
   pvsc_tuning win{256, 0, 0, 1e30f, 0, 0, 0, 0};
   for (const pvsc_tuning& c : cands) {
-    l0->tuning[{R, prec}] = c;
+    install(c);
     drop_graphs(l0);
     const size_t wb = pvsc_batched_work_bytes(lats, n, R, prec, M);
     double* mp = static_cast<double*>(mu);
@@ -604,7 +652,8 @@ int pvsc_autotune_batched(pvsc_lattice* const* lats, int n, int R, int prec, con
     drop_graphs(l0);
     return rc;
   }
-  l0->tuning[{R, prec}] = win;
+  install(win);
+  if (win.threads == 0) win.threads = 256;  // as an untuned entry reads
   drop_graphs(l0);
   if (best) *best = win;
   return PVSC_OK;

@@ -178,6 +178,7 @@ int launch_sweep_shape(const pvsc_lattice* lat, int prec, int feat, Sweep& p, La
     // sixteen warps where the accumulator is read and written (its loads are the longest waits)
     LaunchShape d;
     d.threads = (feat & F_ACC) ? 512 : 256;
+    if (sh.side_by_side) d.zslab = sh.zslab;
     return launch_sweep_tma(lat, feat, p, d, st);
   }
   if (sh.kernel == kKernelTma || sh.kernel == kKernelTmaX) {

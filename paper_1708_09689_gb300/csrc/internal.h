@@ -40,6 +40,7 @@ struct LaunchShape {
                           // 4 two KPM steps per sweep (tile_x x tile_y tiles),
                           // 5 z-marching over tile_x x tile_y column tiles, 6 marching along x,
                           // 7 TMA-staged plane tiles (warp-specialised)
+  bool side_by_side = false;  // one of several sweeps that run at once: zslab holds for an untuned sweep too
   bool tuned = false;     // the fields above are a tuning entry's; else the library's own choice
 };
 
@@ -114,6 +115,7 @@ int launch_sweep_tma_fx(const pvsc_lattice* lat, Sweep& p, const LaunchShape& sh
 int tma_error_fx(int clear, int* flag);
 bool tma_tile_valid(int R, int tile_x, int tile_y);  // (0, 0) or one of the two tiles of this R
 bool tma_tile_deep(int R, int tile_y);
+int64_t tma_large_tiles(const pvsc_lattice* lat, int R);  // large tiles of a plane (times the slices of R = 32, 64)
 int launch_kpm2_sweep(const pvsc_lattice* lat, Sweep& p, const LaunchShape& sh, cudaStream_t st);
 int kpm2_check_tile(int TX, int TY, int R);
 

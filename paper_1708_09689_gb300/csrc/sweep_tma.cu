@@ -78,6 +78,13 @@ static void tma_tiles_of(int R, int* tx_large, int* ty_large, int* tx_deep, int*
   }
 }
 
+int64_t tma_large_tiles(const pvsc_lattice* lat, int R) {
+  int tx, ty, dx, dy;
+  tma_tiles_of(R, &tx, &ty, &dx, &dy);
+  const int64_t Lx = lat->g.model == PVSC_WSM ? lat->g.L[0] / 2 : lat->g.L[0];
+  return ((Lx + tx - 1) / tx) * ((lat->g.L[1] + ty - 1) / ty) * (R > 16 ? R / 16 : 1);
+}
+
 bool tma_tile_deep(int R, int tile_y) {
   int a, b, c, d;
   tma_tiles_of(R, &a, &b, &c, &d);
