@@ -184,6 +184,10 @@ __device__ __forceinline__ double2* acc_ptr(double2* base, int64_t s, int o, int
   return base + ((s * 4 + o) * (int64_t)R + r);
 }
 
+}  // namespace pvsc
+#include "hop_int.cuh"
+namespace pvsc {
+
 // ---------------------------------------------------------------- per-thread constants
 template <typename T, int VPT>
 struct VecCoef {
@@ -893,13 +897,13 @@ __device__ __forceinline__ void hop_y_add(const Blk<double, 1>& a, const Blk<dou
   H.v[3][0] = caddi(H.v[3][0], csub(g0, h0));
 }
 
-// y_new = kt H + d x + gamma y_in from the hopping sum H, complex128 (REC: gamma = -1, two
-// fused operations a part).  yi: zeros in a sweep without y_in (a branch on it becomes predicated
+// y_new = kt H + d x + gamma y_in from the hopping sum H, complex128 (kt per real part; REC: gamma
+// = -1, two fused operations a part).  yi: zeros in a sweep without y_in (a branch on it becomes predicated
 // fp64 instructions)
 template <bool REC>
 __device__ __forceinline__ void ti_combine_hop(const VecCoef<double, 1>& cf, double Vs, const Blk<double, 1>& xc,
-                                               const Blk<double, 1>& H, const Blk<double, 1>* yi,
-                                               Blk<double, 1>& yn) {
+                                               const Blk<double, 1>& H, const double (&kt)[8],
+                                               const Blk<double, 1>* yi, Blk<double, 1>& yn) {
   const double dp = fma(cf.alpha[0], Vs, cf.am[0] - cf.ab[0]), dm = fma(cf.alpha[0], Vs, -cf.am[0] - cf.ab[0]);
 #pragma unroll
   for (int o = 0; o < 4; ++o) {
@@ -911,15 +915,39 @@ __device__ __forceinline__ void ti_combine_hop(const VecCoef<double, 1>& cf, dou
     } else {
       t = {fma(cf.gamma[0], yi->v[o][0].re, dd * x.re), fma(cf.gamma[0], yi->v[o][0].im, dd * x.im)};
     }
-    yn.v[o][0] = {fma(cf.kt[0], H.v[o][0].re, t.re), fma(cf.kt[0], H.v[o][0].im, t.im)};
+    yn.v[o][0] = {fma(kt[2 * o], H.v[o][0].re, t.re), fma(kt[2 * o + 1], H.v[o][0].im, t.im)};
+  }
+}
+
+// The hopping sum and the factor kt in its units, part by part, from the neighbour blocks that
+// get(axis, a, b) gives (hop_int): on the integer pipes, or where a part's exponent is out of their
+// range in fp64.
+template <bool RELOAD, class Get>
+__device__ __forceinline__ void ti_hop(double kt, Get&& get, Blk<double, 1>& H, double (&kth)[8]) {
+  int off[8];
+  if (hop_int_factor(kt) && hop_int<RELOAD>(get, H, off)) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) kth[i] = __hiloint2double(__double2hiint(kt) + off[i], __double2loint(kt));
+  } else {
+    Blk<double, 1> a, b;
+    get(0, a, b);
+    hop_z_init(a, b, H);
+    get(1, a, b);
+    hop_x_add(a, b, H);
+    get(2, a, b);
+    hop_y_add(a, b, H);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) kth[i] = kt;
   }
 }
 
 // y_new of one TI site from the blocks around it (Delta terms aside).  complex64 folds S and
-// D (ti_axes, ti_combine_core).  complex128 is bound by the fp64 pipe of this part (1/64 of
-// the fp32 rate: two lanes per SM), so it takes the projected hopping sum and the shortest
-// update.  100 fp64 operations per site and vector with two dot
-// products, from 133 with S and D.
+// D (ti_axes, ti_combine_core).  complex128 is bound by the fp64 pipe of this part (1/64 of the
+// fp32 rate: two lanes per SM), so its hopping sum goes over the integer pipes (hop_int) and its
+// update is the shortest: 45 fp64 instructions per site and vector with two dot products (100
+// with the projected fp64 sum, 133 with S and D).  KPM sweep of 128x128x64, R = 8: 1.59 ms with
+// the fp64 sum, 1.03 ms so (1170 ALU instructions a value; fp64 pipe 60 % and ALU 50 % busy with the
+// eight warps of the register march).
 template <bool REC, typename T, int VPT>
 __device__ __forceinline__ void ti_update(const VecCoef<T, VPT>& cf, T Vs, const Blk<T, VPT>& zm,
                                           const Blk<T, VPT>& xc, const Blk<T, VPT>& zp, const Blk<T, VPT>& xm,
@@ -927,10 +955,12 @@ __device__ __forceinline__ void ti_update(const VecCoef<T, VPT>& cf, T Vs, const
                                           const Blk<T, VPT>* yi, Blk<T, VPT>& yn) {
   if constexpr (sizeof(T) == 8) {
     Blk<double, 1> H;
-    hop_z_init(zm, zp, H);
-    hop_x_add(xm, xp, H);
-    hop_y_add(ym, yp, H);
-    ti_combine_hop<REC>(cf, Vs, xc, H, yi, yn);
+    double kt[8];
+    ti_hop<false>(cf.kt[0], [&](int axis, Blk<double, 1>& a, Blk<double, 1>& b) {
+      a = axis == 0 ? zm : (axis == 1 ? xm : ym);
+      b = axis == 0 ? zp : (axis == 1 ? xp : yp);
+    }, H, kt);
+    ti_combine_hop<REC>(cf, Vs, xc, H, kt, yi, yn);
   } else {
     Blk<T, VPT> S, D;
     ti_axes(zm, zp, xm, xp, ym, yp, S, D);
