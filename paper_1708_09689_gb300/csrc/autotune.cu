@@ -68,9 +68,10 @@ static void cache_store(const std::string& key, const pvsc_tuning& t) {
 }
 
 // The untuned sweep as a candidate, where no tuning entry can select it (the TMA-staged tiles of a
-// lattice with Lx no multiple of 4): threads = 0 stands for it in the list and in the cache file,
+// lattice with Lx no multiple of 4, and of complex128 vectors): threads = 0 stands for it in the list and in the cache file,
 // and installing it removes the entry.  The caller is told the defaults that pvsc_get_tuning reads.
 static bool untuned_is_its_own(const pvsc_lattice* lat, int R, int prec) {
+  if (prec == PVSC_C128) return tma_c128_default(lat, R);
   return tma_sweep_default(lat, R, prec) && !tma_sweep_possible(lat, R, prec);
 }
 

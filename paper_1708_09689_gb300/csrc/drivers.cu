@@ -174,6 +174,8 @@ int launch_sweep_shape(const pvsc_lattice* lat, int prec, int feat, Sweep& p, La
     sh = LaunchShape{};
     sh.zslab = zs;
   }
+  if (!sh.tuned && prec == PVSC_C128 && !(feat & F_ADJ) && tma_c128_default(lat, p.R))
+    return launch_sweep_tma_c128(lat, feat, p, st);
   if (!sh.tuned && !(feat & F_ADJ) && tma_sweep_default(lat, p.R, prec)) {
     // sixteen warps where the accumulator is read and written (its loads are the longest waits)
     LaunchShape d;

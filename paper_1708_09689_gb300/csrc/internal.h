@@ -54,6 +54,7 @@ constexpr int kModelWSMMarch = 9;    // Weyl semimetal z-marching cell sweep
 constexpr int kModelGrapheneQD = 10; // graphene sweep with the regenerated quantum-dot array
 constexpr int kModelTIXMarch = 11;   // TI sweep marching along x (tuning kernel 6)
 constexpr int kModelTIFx = 12;       // TI KPM sweep on fixed-point (PVSC_Q64) vectors
+constexpr int kModelTIC128 = 13;     // TI sweep on complex128 vectors, TMA-staged tiles
 constexpr int kAsyncDepth = 1;
 constexpr int kAsyncDeepDepth = 3;
 // ring: (depth + 1) slots x buffers x 4 granules of 16 bytes per thread
@@ -113,6 +114,10 @@ int tma_error(int clear, int* flag);
 bool tma_fx_possible(const pvsc_lattice* lat, int R);
 int launch_sweep_tma_fx(const pvsc_lattice* lat, Sweep& p, const LaunchShape& sh, cudaStream_t st);
 int tma_error_fx(int clear, int* flag);
+// complex128 TI sweeps on TMA-staged tiles (sweep_tma_c128.cu), the choice of untuned sweeps
+bool tma_c128_default(const pvsc_lattice* lat, int R);
+int launch_sweep_tma_c128(const pvsc_lattice* lat, int feat, Sweep& p, cudaStream_t st);
+int tma_error_c128(int clear, int* flag);
 bool tma_tile_valid(int R, int tile_x, int tile_y);  // (0, 0) or one of the two tiles of this R
 bool tma_tile_deep(int R, int tile_y);
 int64_t tma_large_tiles(const pvsc_lattice* lat, int R);  // large tiles of a plane (times the slices of R = 32, 64)

@@ -152,7 +152,9 @@ int tma_error(int clear, int* flag) {
   if (int rc = tma_error_fx(clear, &c)) return rc;
   if (int rc = tma_error_sliced(clear, &d)) return rc;
   if (int rc = tma_error_xm(clear, &e)) return rc;
-  *flag = (a || b || c || d || e || f) ? 1 : 0;
+  int h = 0;
+  if (int rc = tma_error_c128(clear, &h)) return rc;
+  *flag = (a || b || c || d || e || f || h) ? 1 : 0;
   return PVSC_OK;
 }
 

@@ -246,18 +246,20 @@ __device__ __forceinline__ void tma_lds_blk(const unsigned char* buf, uint32_t B
   b.v[3][0] = {v1.z, v1.w};
 }
 
-// The same four orbitals of a fixed-point block: a site of R/2 vectors of
-// 16-byte (re, im) 64-bit pairs has the byte layout of a complex64 site of R
+// The same four orbitals of a fixed-point or complex128 block: a site of R/2
+// vectors of 16-byte (re, im) 64-bit pairs has the byte layout of a complex64 site of R
 // vectors, and vector c is the 16-byte chunk c of every orbital.  SWZ = false
 // (unswizzled tiles): orbital o at B + its offset, an immediate of the load.
-template <int R, bool SWZ = true>
-__device__ __forceinline__ void tma_lds_blk(const unsigned char* buf, uint32_t B, Blk<long long, 1>& b) {
+template <int R, bool SWZ = true, typename E>
+__device__ __forceinline__ void tma_lds_blk(const unsigned char* buf, uint32_t B, Blk<E, 1>& b) {
+  static_assert(sizeof(E) == 8, "16-byte values");
+  using P2 = typename Pair16<E>::type;
 #pragma unroll
   for (int o = 0; o < 4; ++o) {
     const int ao = o * 8 * R;
     const int K1 = (ao >> 4) & 7, K2 = (ao >> 7) & 7;
     const uint32_t off = SWZ ? (B ^ (uint32_t)((K1 ^ K2) << 4)) + (uint32_t)(ao & ~127) : B + (uint32_t)ao;
-    const longlong2 v = *reinterpret_cast<const longlong2*>(buf + off);
+    const P2 v = *reinterpret_cast<const P2*>(buf + off);
     b.v[o][0] = {v.x, v.y};
   }
 }
@@ -267,7 +269,9 @@ __device__ __forceinline__ void tma_lds_blk(const unsigned char* buf, uint32_t B
 // the cell update of the Weyl sweeps and two potentials per cell;
 // kModelTIFx: the TI KPM sweep of sweep_fx.cu on fixed-point vectors (R/2
 // vectors in the byte layout of R complex64 vectors, one vector per thread,
-// the per-site coefficient pair in place of the potential, exact dot sums).
+// the per-site coefficient pair in place of the potential, exact dot sums);
+// kModelTIC128: TI sites of complex128 vectors in the same layout (R/2 vectors,
+// one per thread), the arithmetic of ti_update, the fp64 potential.
 // SL > 1: the block of R SL vectors is swept as SL slices of R vectors
 // (R = 16, the layout of the 8 x 8 tiles): block b takes slice b mod SL
 // (the grid is a multiple of SL), whose 128-byte rows the tensor maps select
@@ -285,14 +289,16 @@ __global__ void __launch_bounds__(32 * NW, 1)
   static_assert(SL == 1 || R == 16, "vector slices of 16 complex64 (8 fixed-point) vectors");
   static_assert(!XM || MODEL == PVSC_TI || MODEL == PVSC_WSM, "marching along x: TI sites or Weyl cells");
   constexpr int RF = R * SL;  // vectors (complex64 layout) of the whole block
-  constexpr int VP = R == 1 ? 1 : 2;  // complex64 vectors per thread (R = 1: one per site)
   constexpr bool WSM = MODEL == 3;
   constexpr bool FX = MODEL == kModelTIFx;
-  // fixed point with R/2 >= 8 vectors: a quarter-warp reads one whole 128-byte
+  constexpr bool CD = MODEL == kModelTIC128;
+  using T = typename std::conditional<CD, double, float>::type;  // arithmetic (not fixed point)
+  constexpr int VP = (R == 1 || CD) ? 1 : 2;  // vectors per thread (complex64 R = 1: one per site)
+  // 16-byte values, R/2 >= 8 vectors: a quarter-warp reads one whole 128-byte
   // row of an orbital, conflict-free without the swizzle (no XOR per load)
-  constexpr bool SWZ = !(FX && R >= 16);
+  constexpr bool SWZ = !((FX || CD) && R >= 16);
   constexpr int VPC = WSM ? 2 : 1;               // sites per tile point
-  constexpr int VF = WSM ? 2 : (FX ? 4 : 1);     // 4-byte words of potential data per tile point
+  constexpr int VF = (WSM || CD) ? 2 : (FX ? 4 : 1);  // 4-byte words of potential data per tile point
   using L = TmaLayout<R, DEEP, NW, FX ? 4 : 2>;
   constexpr int NCW = NW, IPT = L::IPT, TX = L::TX, TY = L::TY;
   extern __shared__ unsigned char smem_raw[];
@@ -486,12 +492,11 @@ __global__ void __launch_bounds__(32 * NW, 1)
   const int c = lane % L::CPS;
   const int q = lane / L::CPS;
   const int cg = c + sl * L::CPS;  // the chunk (complex64) or vector (fixed point) in the block
-  VecCoef<float, VP> cf;
-  if constexpr (!FX) {
-    cf = load_coef<float, VP>(p, cg);
-    hold_coef(cf);
-  }
-  DotAcc<float, VP> dacc;  // compensated fp32 sums; their fp64 part lives in shared memory
+  VecCoef<T, VP> cf;
+  if constexpr (!FX) cf = load_coef<T, VP>(p, cg);
+  if constexpr (!FX && !CD) hold_coef(cf);
+  // complex64: compensated fp32 sums, their fp64 part in shared memory; complex128: fp64 sums of a unit
+  DotAcc<T, VP> dacc;
   dacc.init();
   // fixed point: exact per-unit dot sums of this thread's vector c, the
   // coefficient limbs and the fp64 value of one dot unit
@@ -526,14 +531,20 @@ __global__ void __launch_bounds__(32 * NW, 1)
     for (int d = 0; d < num_dots(FEAT); ++d)
 #pragma unroll
       for (int v = 0; v < VP; ++v) {
-        double t = widen(dacc.s[d][v]) + widen(dacc.c[d][v]);
-        dacc.s[d][v] = 0.f;
-        dacc.c[d][v] = 0.f;
+        double t;
+        if constexpr (CD) {
+          t = dacc.d[d][v];
+          dacc.d[d][v] = 0.0;
+        } else {
+          t = widen(dacc.s[d][v]) + widen(dacc.c[d][v]);
+          dacc.s[d][v] = 0.f;
+          dacc.c[d][v] = 0.f;
+        }
         for (int off = 16; off >= L::CPS; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
         if (lane < L::CPS) wdots[(d * 2 + v) * L::CPS + lane] += t;
       }
   };
-  using XBlk = typename std::conditional<FX, Blk<long long, 1>, Blk<float, VP>>::type;
+  using XBlk = typename std::conditional<FX, Blk<long long, 1>, Blk<T, VP>>::type;
   XBlk xmr[IPT];
   uint32_t kx = 0, ky = 0;
   const unsigned char* ybase = base + L::NXS * L::XSTAGE;
@@ -570,7 +581,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
 #pragma unroll
       for (int i = 0; i < IPT; ++i)
         if (ok[i]) {
-          if constexpr (FX)
+          if constexpr (FX || CD)
             tma_lds_blk<R, SWZ>(s0, Bc[i], xmr[i]);
           else
             tma_lds_blk<R>(s0, Bc[i], xmr[i]);
@@ -600,13 +611,14 @@ __global__ void __launch_bounds__(32 * NW, 1)
           // the accumulator (and source) lines of this site two planes ahead into
           // L2, so that the epilogue's fp64 reads do not wait on HBM; one thread
           // per 128-byte line of its chunks
-          if (z + 2 < Lz && (cg & 3) == 0) {
+          constexpr int RV = CD ? RF / 2 : RF, LINE = CD ? 8 : 4;  // vectors of a row, chunks of a line
+          if (z + 2 < Lz && (cg & (LINE - 1)) == 0) {
             const int64_t s2 = s + 2 * plane;
             const bool rd = !(p.acc_mode & ACC_INIT), rs = (p.acc_mode & ACC_XSRC) != 0;
 #pragma unroll
             for (int o = 0; o < 4; ++o) {
-              if (rd) prefetch_l2(acc_ptr(p.acc, s2, o, RF, 2 * cg));
-              if (rs) prefetch_l2(acc_ptr(const_cast<double2*>(p.src), s2, o, RF, 2 * cg));
+              if (rd) prefetch_l2(acc_ptr(p.acc, s2, o, RV, (CD ? 1 : 2) * cg));
+              if (rs) prefetch_l2(acc_ptr(const_cast<double2*>(p.src), s2, o, RV, (CD ? 1 : 2) * cg));
             }
           }
         }
@@ -655,6 +667,28 @@ __global__ void __launch_bounds__(32 * NW, 1)
           }
           store_blk<long long, 1>(static_cast<long long*>(p.yout), s, RF / 2, cg, yn);
           fx_dot_item(xs, ys, fxx, fxy);
+          xmr[i] = xc;
+        } else if constexpr (CD) {
+          // ti_update, the neighbours read from the tiles where they are needed (twice)
+          Blk<double, 1> H, xc, yi, yn;
+          double kt[8];
+          ti_hop<true>(cf.kt[0], [&](int axis, Blk<double, 1>& a, Blk<double, 1>& b) {
+            if (axis == 0) {
+              a = xmr[i];
+              tma_lds_blk<R, SWZ>(s1, Bc[i], b);
+            } else {
+              tma_lds_blk<R, SWZ>(s0, axis == 1 ? Bxm[i] : Bym[i], a);
+              tma_lds_blk<R, SWZ>(s0, axis == 1 ? Bxp[i] : Byp[i], b);
+            }
+          }, H, kt);
+          tma_lds_blk<R, SWZ>(s0, Bc[i], xc);
+          if (m.has_yin) tma_lds_blk<R, SWZ>(sy, Bc[i], yi);
+          else zero_blk(yi);
+          const double Vs = m.v_tma ? *reinterpret_cast<const double*>(sy + Vo[i]) : site_potential(g, s);
+          ti_combine_hop<is_recurrence(FEAT)>(cf, Vs, xc, H, kt, &yi, yn);
+          if (g.has_delta) ti_add_delta(g, cf, xc, yn);
+          const int64_t sites[4] = {s, s, s, s};
+          epilogue<double, 1, FEAT>(p, s, cg, xc, yn, dacc, sites, yi);
           xmr[i] = xc;
         } else {
           if constexpr (WSM) {
@@ -760,7 +794,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
     // blocks in finish_dots (after an abort the values are garbage, but the
     // arrival counter stays consistent)
     const double* wd = reinterpret_cast<const double*>(base + L::DOT_OFF);
-    constexpr int RV = FX ? R / 2 : R;  // vectors of a slice
+    constexpr int RV = (FX || CD) ? R / 2 : R;  // vectors of a slice
     constexpr int RVF = RV * SL;        // of the block (this block writes its slice's)
     double* row = p.partials + (size_t)blockIdx.x * p.row_len;
     constexpr int ND = FX ? 2 : num_dots(FEAT);
@@ -769,6 +803,8 @@ __global__ void __launch_bounds__(32 * NW, 1)
       double sum = 0.0;
       if constexpr (FX) {
         for (int w = 0; w < NCW; ++w) sum += wd[w * kNumDots * 2 * L::CPS + d * L::CPS + r];
+      } else if constexpr (CD) {
+        for (int w = 0; w < NCW; ++w) sum += wd[(w * kNumDots + d) * 2 * L::CPS + r];
       } else {
         for (int w = 0; w < NCW; ++w) sum += wd[((w * kNumDots + d) * 2 + (r & 1)) * L::CPS + (r >> 1)];
       }
@@ -801,7 +837,8 @@ static int encode_maps(const pvsc_lattice* lat, const Sweep& p, TmaMaps& m) {
   const int vpc = lat->g.model == PVSC_WSM ? 2 : 1;  // Weyl cells: two sites each
   // 4-byte words of potential data per tile point: fp32 potentials, or the
   // fixed-point sweep's per-site (d+, d-) pair of 64-bit coefficients
-  const int vf = MODEL == kModelTIFx ? 4 : vpc;
+  // or fp64 potentials
+  const int vf = MODEL == kModelTIFx ? 4 : (MODEL == kModelTIC128 ? 2 : vpc);
   const cuuint64_t Lx = lat->g.L[0] / vpc, Ly = lat->g.L[1], Lz = lat->g.L[2];
   // rows of ROWB bytes (128; a whole 64- or 32-byte site for R = 2, 1); with SL
   // slices a row of the block holds SL slice rows side by side (the innermost
@@ -814,8 +851,8 @@ static int encode_maps(const pvsc_lattice* lat, const Sweep& p, TmaMaps& m) {
                                  XM ? SB : SB * Lx * Ly};
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   // the kernel's addressing: the swizzle spanning a row (128, 64 or 32 bytes);
-  // unswizzled tiles for fixed point with R/2 >= 8 vectors
-  const CUtensorMapSwizzle swz = (MODEL == kModelTIFx && R >= 16) ? CU_TENSOR_MAP_SWIZZLE_NONE
+  // unswizzled tiles for 16-byte values with R/2 >= 8 vectors
+  const CUtensorMapSwizzle swz = ((MODEL == kModelTIFx || MODEL == kModelTIC128) && R >= 16) ? CU_TENSOR_MAP_SWIZZLE_NONE
                                  : L::ROWB == 128                 ? CU_TENSOR_MAP_SWIZZLE_128B
                                  : L::ROWB == 64                  ? CU_TENSOR_MAP_SWIZZLE_64B
                                                                   : CU_TENSOR_MAP_SWIZZLE_32B;
@@ -835,14 +872,17 @@ static int encode_maps(const pvsc_lattice* lat, const Sweep& p, TmaMaps& m) {
   if (m.has_yin)
     if (int rc = tile5(&m.yi, p.yin, L::TX, L::TY)) return rc;
   m.v_tma = MODEL == kModelTIFx ? 1 : (!XM && lat->g.v_mode == 1);
+  if (MODEL == kModelTIC128 && Lx % 2) m.v_tma = 0;  // rows of 8 Lx bytes: the copy wants 16-byte strides
   if (m.v_tma) {
     // rows of 4-byte words, in the padded copy where Lx is no multiple of 4 (16-byte strides)
-    const bool padded = MODEL != kModelTIFx && lat->g.L[0] % 4 != 0;
+    const bool padded = MODEL != kModelTIFx && MODEL != kModelTIC128 && lat->g.L[0] % 4 != 0;
     const cuuint64_t pitch = padded ? 4 * padded_row(lat->g.L[0]) : 4 * vf * Lx;
     const cuuint64_t vd[3] = {vf * Lx, Ly, Lz};  // per site
     const cuuint64_t vs[2] = {pitch, pitch * Ly};
     const cuuint32_t vb[3] = {(cuuint32_t)(vf * L::TX), (cuuint32_t)L::TY, 1};
-    void* vptr = MODEL == kModelTIFx ? const_cast<void*>(p.fx_d) : static_cast<void*>(padded ? lat->V32p_dev : lat->V32_dev);
+    void* vptr = MODEL == kModelTIFx     ? const_cast<void*>(p.fx_d)
+                 : MODEL == kModelTIC128 ? static_cast<void*>(lat->V_dev)
+                                         : static_cast<void*>(padded ? lat->V32p_dev : lat->V32_dev);
     const CUresult r = enc(&m.v, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, vptr, vd, vs, vb,
                            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -866,7 +906,10 @@ static void* tma_kernel(int feat) {
     }
   } else {
     switch (feat) {
-      case F_REC:  // the same arithmetic in fp32
+      case F_REC:
+        if constexpr (MODEL == kModelTIC128)
+          return reinterpret_cast<void*>(&ti_sweep_tma<R, DEEP, NW, F_REC, MODEL, SL>);
+        [[fallthrough]];  // the same arithmetic in fp32
       case 0: return reinterpret_cast<void*>(&ti_sweep_tma<R, DEEP, NW, 0, MODEL, SL>);
       case F_DOTS: return reinterpret_cast<void*>(&ti_sweep_tma<R, DEEP, NW, F_DOTS, MODEL, SL>);
       case F_KPM: return reinterpret_cast<void*>(&ti_sweep_tma<R, DEEP, NW, F_KPM, MODEL, SL>);

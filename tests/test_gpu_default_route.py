@@ -52,6 +52,34 @@ def test_default_sweeps_equal_the_march(dims, per, R, model, pot):
     assert pv.device_error() == 0
 
 
+# at least 2^20 site-vectors; odd Lx (potential read per site), remainders, slices of 8 vectors
+@pytest.mark.parametrize("dims,per,R", [((61, 45, 30), (1, 0, 1), 16), ((50, 33, 51), (0, 1, 0), 32),
+                                        ((127, 96, 7), (1, 1, 0), 64), ((90, 72, 41), (0, 0, 1), 4),
+                                        ((66, 64, 33), (1, 1, 1), 8), ((129, 128, 66), (0, 1, 1), 1),
+                                        ((112, 96, 50), (1, 0, 0), 2)])
+@pytest.mark.parametrize("pot", ["stored", "none", "hashed"])
+def test_default_complex128_sweeps_equal_the_march(dims, per, R, pot):
+    lat, ref = _lattice("ti", dims, per, pot), _lattice("ti", dims, per, pot)
+    ref.set_tuning(R, pv.C128, threads=128, kernel=0)
+    x = pv.random_vectors(lat, R, pv.C128, 1)
+    y = pv.random_vectors(lat, R, pv.C128, 2)
+    z = pv.random_vectors(lat, R, pv.C128, 3)
+    out = []
+    for l in (lat, ref):
+        h = pv.apply_H(l, x)
+        y1, z1 = y.clone(), z.clone()
+        d = pv.cheb_step(l, x, y1, [0.2] * R, [0.1] * R, [-0.7] * R, z1, [0.3] * R, dots=7)
+        f = pv.cheb_series(l, x, [0.5, 0.3j, 0.2, 0.1, -0.4 + 0.1j, 0.6, 0.1], 10.0, 0.1)
+        mu = pv.kpm_moments(l, 9, 10.0, 0.1, r0=x)
+        out.append((h, y1, z1, f, d, mu))
+    a, b = out
+    for k in range(4):
+        assert torch.equal(a[k], b[k]), k
+    assert torch.max(torch.abs(a[4] - b[4])).item() < 1e-12
+    assert torch.max(torch.abs(a[5] - b[5])).item() < 1e-12
+    assert pv.device_error() == 0
+
+
 def test_new_potential_reaches_the_padded_rows():
     dims, R = (61, 45, 30), 4
     lat = pv.Lattice.ti(dims, (1, 0, 1))
