@@ -146,6 +146,21 @@ static int coef_kind(double re, double im) {
   return (im == 0.0 ? 1 : 0) | (re == 0.0 ? 2 : 0);  // 1 real, 2 imaginary, 3 zero, 0 general
 }
 
+// Threads per block of an untuned register sweep: 128 where blocks of 256 leave SMs without a share of
+// the work.  KPM sweeps with 256 -> 128 threads, us: TI complex128 (always: its long fp64 and integer
+// phases also balance better) 16^3 R = 1: 10.1 -> 6.8, 32^3 R = 8: 44.9 -> 35.5, 101x87x53 R = 1: 69 -> 65;
+// TI complex64 16^3 R = 2: 8.2 -> 5.8, 20^3 R = 8: 7.2 -> 8.3, 32^3 R = 1: 6.3 -> 7.2; Weyl complex64
+// 16^3 R = 4: 7.1 -> 5.1, R = 16: 5.6 -> 5.8; Weyl complex128 48^3 R = 1: 21.7 -> 16.9, R = 8: 90 -> 91.
+static int default_threads(const pvsc_lattice* lat, int R, int prec) {
+  const int64_t work = lat->g.n_sites * R;
+  bool narrow = false;
+  if (lat->g.model == PVSC_TI)
+    narrow = prec == PVSC_C128 || (work <= 5 << 13 && (R >= 2 || work <= 1 << 14));
+  else if (lat->g.model == PVSC_WSM)
+    narrow = prec == PVSC_C128 ? work <= 1 << 15 || (R <= 4 && work <= 1 << 18) : R <= 8 && work <= 1 << 16;
+  return narrow ? 128 : 256;
+}
+
 int launch_sweep(const pvsc_lattice* lat, int prec, int feat, Sweep& p, cudaStream_t st) {
   return launch_sweep_shape(lat, prec, feat, p, shape_for(lat, p.R, prec), st);
 }
@@ -196,7 +211,7 @@ int launch_sweep_shape(const pvsc_lattice* lat, int prec, int feat, Sweep& p, La
     return launch_sweep_staged(lat, prec, feat, p, sh, st);
   const int vpt = vpt_tuned(sh.vpt, p.R, prec);
   p.C = p.R / vpt;
-  int threads = sh.threads;
+  int threads = sh.tuned ? sh.threads : default_threads(lat, p.R, prec);
   if (tiled) {  // z-marching sweep over tile_x x tile_y column tiles (checked by pvsc_set_tuning)
     threads = sh.tile_x * sh.tile_y * p.C;
     p.tile_x = sh.tile_x;
