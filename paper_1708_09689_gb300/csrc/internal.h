@@ -239,7 +239,7 @@ inline void drop_graphs(pvsc_lattice* lat) {
   lat->graphs.clear();
 }
 
-// Programmatic dependent launch of the TMA-staged sweeps (on unless
+// Programmatic dependent launch of the TMA-staged and the complex128 graphene sweeps (on unless
 // PVSC_NO_PDL is set to a value other than 0).
 inline bool pdl_enabled() {
   const char* e = std::getenv("PVSC_NO_PDL");

@@ -82,7 +82,18 @@ int launch_sweep_c128(int model, int feat, int grid, int threads, const Sweep& p
   if (smem)
     if (int rc = allow_max_smem(fn)) return rc;
   void* args[] = {const_cast<Sweep*>(&p)};
-  PVSC_CUDA_TRY(cudaLaunchKernel(fn, dim3(grid), dim3(threads), args, smem, st));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  // gr_site_sweep begins with pdl_begin
+  cfg.numAttrs = model == PVSC_GRAPHENE && gr_by_site(feat) && pdl_enabled() ? 1 : 0;
+  PVSC_CUDA_TRY(cudaLaunchKernelExC(&cfg, fn, args));
   return PVSC_OK;
 }
 
