@@ -150,8 +150,10 @@ def _check(rc: int):
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return ctypes.c_void_p(stream.cuda_stream)
+    # the current stream's handle without a Stream object around it (3 us a call)
+    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 def _ptr(t: torch.Tensor | None):
@@ -345,11 +347,18 @@ def apply_H(lat: Lattice, x: torch.Tensor, y: torch.Tensor | None = None, stream
     return y
 
 
+def _dots_out(R: int, dots: int, device) -> torch.Tensor:
+    """The [4, R] output of a step's dot products: zeros where a row stays unwritten (all three flags
+    write all four rows, and a fill is a third of a small step's time)."""
+    make = torch.empty if dots == DOT_XX | DOT_XY | DOT_YY else torch.zeros
+    return make((4, R), dtype=torch.float64, device=device)
+
+
 def cheb_step(lat: Lattice, x, y, alpha, beta, gamma=None, z=None, delta=None, dots: int = 0,
               work: torch.Tensor | None = None, stream=None):
     """y <- alpha (H - beta) x + gamma y; z += delta y; returns the dots tensor [4, R] or None."""
     R, prec = block_R(x), prec_of(x)
-    d = torch.zeros((4, R), dtype=torch.float64, device=x.device) if dots else None
+    d = _dots_out(R, dots, x.device) if dots else None
     if dots and work is None:
         work = work_buffer(lat.work_bytes(OP_CHEB_STEP, R, prec))
     _check(_lib.pvsc_cheb_step(
@@ -366,7 +375,7 @@ def cheb_step_noalloc(lat: Lattice, x, y, alpha, beta, gamma=None, z=None, delta
     device) may be passed in so that this call allocates nothing either."""
     R, prec = block_R(x), prec_of(x)
     if dots and out_dots is None:
-        out_dots = torch.zeros((4, R), dtype=torch.float64, device=x.device)
+        out_dots = _dots_out(R, dots, x.device)
     _check(_lib.pvsc_cheb_step_noalloc(
         lat.handle, R, prec, _ptr(x), _ptr(y), _ptr(z), _darr(alpha), _darr(beta),
         _darr(gamma) if gamma is not None else None, _darr(delta) if delta is not None else None,
