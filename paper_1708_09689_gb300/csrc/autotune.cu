@@ -109,7 +109,6 @@ extern "C" int pvsc_autotune_op(pvsc_lattice* lat, int R, int prec, int op, pvsc
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t vb = vec_bytes(lat, R, prec), wb = dots_work_bytes(lat, R);
   void *x = nullptr, *y = nullptr, *work = nullptr, *acc = nullptr;
-  double* dots = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   int rc = PVSC_OK;
   auto cleanup = [&]() {
@@ -118,13 +117,11 @@ extern "C" int pvsc_autotune_op(pvsc_lattice* lat, int R, int prec, int op, pvsc
     cudaFree(x);
     cudaFree(y);
     cudaFree(work);
-    cudaFree(dots);
     cudaFree(acc);
   };
   const size_t ab = op == PVSC_OP_SERIES ? vec_bytes(lat, R, PVSC_C128) : 16;
   if (cudaMalloc(&x, vb) != cudaSuccess || cudaMalloc(&y, vb) != cudaSuccess ||
-      cudaMalloc(&work, wb) != cudaSuccess || cudaMalloc(&dots, sizeof(double) * 4 * R) != cudaSuccess ||
-      cudaMalloc(&acc, ab) != cudaSuccess) {
+      cudaMalloc(&work, wb) != cudaSuccess || cudaMalloc(&acc, ab) != cudaSuccess) {
     cleanup();
     return set_error(PVSC_ERR_OOM, "autotune could not allocate its sweep vectors");
   }
@@ -171,8 +168,6 @@ extern "C" int pvsc_autotune_op(pvsc_lattice* lat, int R, int prec, int op, pvsc
     p.yout = y;
     p.dot_flags = 3;
     p.dot_mode = 0;
-    p.dots = dots;
-    p.counter = static_cast<unsigned*>(work);
     p.partials = reinterpret_cast<double*>(static_cast<char*>(work) + kWorkHeader);
     p.acc = static_cast<double2*>(acc);
     p.acc_out = static_cast<double2*>(acc);
@@ -180,7 +175,6 @@ extern "C" int pvsc_autotune_op(pvsc_lattice* lat, int R, int prec, int op, pvsc
     p.cx_re = 0.3;  // real weights, the kinds of a filter's three-term touch
     p.cy_re = -0.2;
     p.cz_re = -0.1;
-    PVSC_CUDA_TRY(cudaMemsetAsync(work, 0, kWorkHeader, st));
     auto one = [&]() -> int {
       if (op == PVSC_OP_KPM) return launch_sweep(lat, prec, F_KPM, p, st);
       if (op == PVSC_OP_APPLY) return launch_sweep(lat, prec, 0, p, st);

@@ -267,12 +267,11 @@ struct Sweep {
   double* partials;      // [gridDim][row_len]: a row per block, dot d of vector r at d R + r
   int row_len;           // 4 R; in a chain of KPM sweeps 2 R (two dots)
   int grid_rows;         // set at launch: the rows this sweep writes
-  // a chain of KPM sweeps (kpm_chain): this sweep leaves its rows to the next one (defer), and sums the
-  // prev_rows rows that the one before left (step prev_k; prev_slices as dot_slices)
-  int defer;
+  // a chain of KPM sweeps (kpm_chain): this one sums the prev_rows rows that the one before left (step
+  // prev_k; prev_slices as dot_slices)
   int prev_rows, prev_slices, prev_k;
   const double* prev_partials;
-  unsigned* counter;     // zero before the first sweep; reset by the last block
+  unsigned* counter;     // two-step KPM sweep: zero before the first, reset by the last block
   double* dots;          // [4][R]
   double* mu;            // [R][M]
   int M;
@@ -328,10 +327,10 @@ __device__ __forceinline__ double warp_sum_rows(const double* col, int b0, int s
 
 // The rows that the previous sweep of a KPM chain left: every block takes one value (or, with
 // fewer blocks than values, one per warp) with one warp, beside the block's own first loads.
-// The fence, the counter and the last block's sum (round trips to L2 and a dozen dependent fp64
-// additions) are then off the end of every sweep but the last.  KPM sweeps: Weyl 256x32x32, R = 16
-// (flat) 53.5 -> 44.3 us; 256x64x8, R = 32 (z-march) 116 -> 103 us; 16^3, R = 1, complex128 15.8
-// -> 12.8 us; 256x256x64, R = 8 (kernel 7) 497 -> 488 us.
+// A sweep thus ends with its rows written: the fence, the counter and the last block's sum of a
+// sweep that finishes its own dots (round trips to L2 and a dozen dependent fp64 additions) are off
+// its end.  KPM sweeps: Weyl 256x32x32, R = 16 (flat) 53.5 -> 44.3 us; 256x64x8, R = 32 (z-march)
+// 116 -> 103 us; 16^3, R = 1, complex128 15.8 -> 12.8 us; 256x256x64, R = 8 (kernel 7) 497 -> 488 us.
 __device__ __forceinline__ void finish_prev(const Sweep& p) {
   if (p.prev_rows == 0) return;
   const int nwarps = blockDim.x >> 5, warp = nwarps - 1 - (int)(threadIdx.x >> 5);  // the last warp first
@@ -344,19 +343,9 @@ __device__ __forceinline__ void finish_prev(const Sweep& p) {
   }
 }
 
-// After every block has written its row of `partials`: the last block to
-// arrive sums the rows and writes the outputs of dot_mode (a sweep that defers
-// leaves its rows to finish_prev).  Few values: a warp per value.  More than two
-// values a warp: the whole block takes part, thread t summing value q = t mod nq
-// over every (blockDim / nq)-th row (neighbouring threads on neighbouring
-// values, the loads independent of one another), then the groups as a tree, so
-// that it is about one round trip to L2 whatever R (at R = 32 on a 32x32x32
-// lattice 11 us less than a warp per value).  scratch: shared memory of blockDim
-// doubles that no thread of the block uses any more.  A KPM step reads the
-// first two dots only; with dot_slices > 1 the rows of slice s are those of
-// the blocks b with b mod dot_slices = s.
-__device__ __forceinline__ void finish_dots(const Sweep& p, double* scratch) {
-  if (p.defer) return;
+// The two-step KPM sweep finishes its own dots: after every block has written its row of
+// `partials`, the last block to arrive sums the rows, a warp per value.
+__device__ __forceinline__ void finish_dots(const Sweep& p) {
   __shared__ int s_last;
   __threadfence();
   __syncthreads();
@@ -364,56 +353,17 @@ __device__ __forceinline__ void finish_dots(const Sweep& p, double* scratch) {
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  const int R = p.R, nb = gridDim.x, nthr = blockDim.x, t = threadIdx.x;
-  const bool kpm = p.dot_mode == 1 || p.dot_mode == 2;
-  const int nq = (kpm ? 2 : kNumDots) * R;  // a power of two
-  const int SL = p.dot_slices > 1 ? p.dot_slices : 1;
-  auto wanted = [&](int d) { return ((p.dot_flags >> (d == 0 ? 0 : (d == 3 ? 2 : 1))) & 1) != 0; };
-  // mu_0 or mu_1, loaded beside the rows
-  auto base_of = [&](int d, int r) {
-    return p.dot_mode >= 2 && (d & 1) < p.M ? __ldcg(p.mu + (size_t)r * p.M + (d & 1)) : 0.0;
-  };
-  if (nq <= 2 * (nthr >> 5)) {
-    for (int q = t >> 5; q < nq; q += nthr >> 5) {
-      const int d = q / R, r = q & (R - 1);
-      if (!wanted(d)) continue;
-      const double base = base_of(d, r);
-      const double s = warp_sum_rows(p.partials + q, SL > 1 ? r / (R / SL) : 0, SL, nb, p.row_len);
-      if ((t & 31) == 0) write_dot(p, p.dot_mode, p.kpm_k, d, r, s, base);
-    }
-  } else {
-    const int ng = nthr < nq ? 1 : 1 << (31 - __clz(nthr / nq));  // groups, a power of two
-    for (int q0 = 0; q0 < nq; q0 += nthr) {
-      const int q = ng > 1 ? (t & (nq - 1)) : q0 + t, grp = ng > 1 ? t / nq : 0;
-      const int d = q / R, r = q & (R - 1);
-      const bool on = q < nq && grp < ng && wanted(d);
-      double s = 0.0, base = 0.0;
-      if (on) {
-        if (grp == 0) base = base_of(d, r);
-        const double* col = p.partials + q;
-#pragma unroll 8
-        for (int b = (SL > 1 ? r / (R / SL) : 0) + SL * grp; b < nb; b += SL * ng)
-          s += __ldcg(col + (size_t)b * p.row_len);
-      }
-      if (ng > 1) {
-        scratch[t] = s;
-        __syncthreads();
-        for (int half = ng >> 1; half > 0; half >>= 1) {
-          if (on && grp < half) {
-            s += scratch[t + half * nq];
-            scratch[t] = s;
-          }
-          __syncthreads();
-        }
-      }
-      if (on && grp == 0) write_dot(p, p.dot_mode, p.kpm_k, d, r, s, base);
-    }
+  for (int q = threadIdx.x >> 5; q < kNumDots * p.R; q += blockDim.x >> 5) {
+    const int d = q / p.R, r = q & (p.R - 1);
+    const double base = (d & 1) < p.M ? __ldcg(p.mu + (size_t)r * p.M + (d & 1)) : 0.0;
+    const double s = warp_sum_rows(p.partials + q, 0, 1, gridDim.x, p.row_len);
+    if ((threadIdx.x & 31) == 0) write_dot(p, p.dot_mode, p.kpm_k, d, r, s, base);
   }
   if (threadIdx.x == 0) *p.counter = 0u;
 }
 
 // ND: the dots this sweep forms (a KPM step: the first two; the others' rows stay unwritten
-// and finish_dots does not read them).
+// and are not read).
 template <int VPT, int MAXW = kMaxThreads / 32, int ND = kNumDots>
 __device__ void reduce_dots(const Sweep& p, double (&acc)[kNumDots][VPT]) {
   __shared__ double sm[MAXW][ND][VPT][32];  // [warp][dot][v][lane]
@@ -440,8 +390,6 @@ __device__ void reduce_dots(const Sweep& p, double (&acc)[kNumDots][VPT]) {
     for (int w = w0; w < nwarps; w += stride) s += sm[w][d][v][l];
     row[d * p.R + t * VPT + v] = s;
   }
-  static_assert(MAXW * ND * VPT >= MAXW, "scratch of one double per thread");
-  finish_dots(p, &sm[0][0][0][0]);
 }
 
 

@@ -105,16 +105,15 @@ void sweep_init(Sweep& p, const pvsc_lattice* lat, int R, int prec) {
 }
 
 // A row of a KPM sweep holds two dots where a work buffer has room for four: two buffers of rows.
-void kpm_chain(const pvsc_lattice* lat, Sweep& p, double* partials, int k, bool last) {
+void kpm_chain(const pvsc_lattice* lat, Sweep& p, double* partials, int k) {
   p.row_len = 2 * p.R;
   p.partials = partials + (size_t)(k & 1) * lat->sm_count * kMaxGridPerSM * p.row_len;
   p.kpm_k = k;
   p.dot_mode = k == 0 ? 1 : 2;
-  p.defer = last ? 0 : 1;
 }
 
 void kpm_launched(Sweep& p) {
-  p.prev_rows = p.defer ? p.grid_rows : 0;
+  p.prev_rows = p.grid_rows;
   p.prev_slices = p.dot_slices;
   p.prev_k = p.kpm_k;
   p.prev_partials = p.partials;
@@ -514,7 +513,7 @@ int kpm_enqueue(const pvsc_lattice* lat, int R, int prec, const void* r0, uint64
   const int64_t D = lat->g.n_sites * orbitals_of(lat->g.model);
   const LaunchShape sh = force ? *force : shape_for(lat, R, prec);
   const bool two = !force && kpm2_selected(lat, R, prec);
-  PVSC_CUDA_TRY(cudaMemsetAsync(work, 0, kWorkHeader, cs));
+  if (two) PVSC_CUDA_TRY(cudaMemsetAsync(work, 0, kWorkHeader, cs));
   const void* x0 = r0;
   if (!r0) {
     if (int rc = launch_random_phase(wa, prec, D, R, seed, cs)) return rc;
@@ -538,9 +537,11 @@ int kpm_enqueue(const pvsc_lattice* lat, int R, int prec, const void* r0, uint64
   p.yin = nullptr;
   p.yout = wb;
   p.dot_mode = 1;
-  if (!two) kpm_chain(lat, p, rows, 0, nsteps == 1);  // two steps per sweep: four dots a row, no chain
+  // two steps per sweep: four dots a row and no chain
+  if (!two) kpm_chain(lat, p, rows, 0);
   if (int rc = launch_sweep_shape(lat, prec, F_KPM, p, sh, cs)) return rc;
   if (!two) kpm_launched(p);
+  else if (int rc = launch_sum_rows(p, cs)) return rc;
   const void* prev = x0;
   void* cur = wb;
   for (int r = 0; r < R; ++r) {
@@ -571,20 +572,21 @@ int kpm_enqueue(const pvsc_lattice* lat, int R, int prec, const void* r0, uint64
     p.dot_flags = 3;
     p.yout2 = nullptr;
   }
-  p.dot_mode = 2;
   for (; k < nsteps; ++k) {
     void* out = (r0 && prev == r0) ? (cur == wa ? wb : wa) : const_cast<void*>(prev);
     p.x = cur;
     p.yin = prev;
     p.yout = out;
     p.kpm_k = k;
-    if (!two) kpm_chain(lat, p, rows, k, k == nsteps - 1);
+    p.dot_mode = 2;
+    if (!two) kpm_chain(lat, p, rows, k);
     if (int rc = launch_sweep_shape(lat, prec, F_KPM, p, sh, cs)) return rc;
     if (!two) kpm_launched(p);
+    else if (int rc = launch_sum_rows(p, cs)) return rc;
     prev = cur;
     cur = out;
   }
-  return PVSC_OK;
+  return two ? PVSC_OK : launch_sum_rows(p, cs);
 }
 
 }  // namespace pvsc
@@ -675,11 +677,10 @@ int pvsc_cheb_step(const pvsc_lattice* lat, int R, int prec, const void* x, void
     p.dot_flags = dot_flags;
     p.dot_mode = 0;
     p.dots = dots;
-    p.counter = reinterpret_cast<unsigned*>(work);
     p.partials = reinterpret_cast<double*>(wptr(work, kWorkHeader));
-    PVSC_CUDA_TRY(cudaMemsetAsync(work, 0, kWorkHeader, st));
   }
-  return launch_sweep(lat, prec, feat, p, st);
+  if (int rc = launch_sweep(lat, prec, feat, p, st)) return rc;
+  return dot_flags ? launch_sum_rows(p, st) : PVSC_OK;
 }
 
 // KPM with fixed-point vectors (sweep_fx.cu); TI lattices only.
@@ -735,14 +736,12 @@ static int kpm_moments_fx(const pvsc_lattice* lat, int R, const void* r0, uint64
   const LaunchShape sh = shape_for(lat, R, PVSC_Q64);
   const bool tuned = lat->tuning.count({R, PVSC_Q64}) != 0;
   auto body = [&](cudaStream_t cs) -> int {
-    PVSC_CUDA_TRY(cudaMemsetAsync(work, 0, kWorkHeader, cs));
     if (int rc = launch_fx_prepare(lat, R, r0, seed, a, b, work, L, cs)) return rc;
     void* wa = wptr(work, L.wa);
     void* wb = wptr(work, L.wb);
     Sweep p;
     sweep_init(p, lat, R, PVSC_C128);
     p.C = R;
-    p.counter = reinterpret_cast<unsigned*>(work);
     double* const rows = reinterpret_cast<double*>(wptr(work, kWorkHeader));
     p.mu = mu;
     p.M = M;
@@ -753,7 +752,7 @@ static int kpm_moments_fx(const pvsc_lattice* lat, int R, const void* r0, uint64
     p.x = wa;
     p.yin = nullptr;
     p.yout = wb;
-    kpm_chain(lat, p, rows, 0, nsteps == 1);
+    kpm_chain(lat, p, rows, 0);
     p.fx_dshift = 0;
     p.fx_kt = std::llrint(std::ldexp(-0.5 * lat->g.t / a, 60));
     if (int rc = launch_sweep_fx(lat, p, sh, tuned, cs)) return rc;
@@ -766,12 +765,12 @@ static int kpm_moments_fx(const pvsc_lattice* lat, int R, const void* r0, uint64
       p.x = cur;
       p.yin = prev;
       p.yout = prev;  // w_{k+1} overwrites w_{k-1} element by element
-      kpm_chain(lat, p, rows, k, k == nsteps - 1);
+      kpm_chain(lat, p, rows, k);
       if (int rc = launch_sweep_fx(lat, p, sh, tuned, cs)) return rc;
       kpm_launched(p);
       std::swap(prev, cur);
     }
-    return PVSC_OK;
+    return launch_sum_rows(p, cs);
   };
   return run_graph(lat, key, st, body);
 }
@@ -821,10 +820,8 @@ int pvsc_kpm_sweeps(const pvsc_lattice* lat, int R, int prec, int k_begin, int k
   if (int rc = check_work(work, work_bytes, dots_work_bytes(lat, R))) return rc;
   if (k_end == k_begin) return PVSC_OK;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  PVSC_CUDA_TRY(cudaMemsetAsync(work, 0, kWorkHeader, st));
   Sweep p;
   sweep_init(p, lat, R, prec);
-  p.counter = reinterpret_cast<unsigned*>(work);
   p.partials = reinterpret_cast<double*>(wptr(work, kWorkHeader));
   p.mu = mu;
   p.M = M;
@@ -840,11 +837,11 @@ int pvsc_kpm_sweeps(const pvsc_lattice* lat, int R, int prec, int k_begin, int k
     p.x = wk;
     p.yin = k == 0 ? nullptr : other;
     p.yout = other;
-    kpm_chain(lat, p, reinterpret_cast<double*>(wptr(work, kWorkHeader)), k, k == k_end - 1);
+    kpm_chain(lat, p, reinterpret_cast<double*>(wptr(work, kWorkHeader)), k);
     if (int rc = launch_sweep(lat, prec, F_KPM, p, st)) return rc;
     kpm_launched(p);
   }
-  return PVSC_OK;
+  return launch_sum_rows(p, st);
 }
 
 int pvsc_debug_series_plan(int K, int* terms) {

@@ -183,15 +183,16 @@ int check_ptr(const void* p, const char* name);
 // Fill p.g / p.R / p.C from the lattice; the caller sets the rest.
 void sweep_init(Sweep& p, const pvsc_lattice* lat, int R, int prec);
 // Launch one fused sweep (feat: F_* mask).  Dot features need p.partials and
-// p.counter inside a work buffer of at least dots_work_bytes(lat, R) bytes.
+// a work buffer of at least dots_work_bytes(lat, R) bytes, and leave rows.
 int launch_sweep(const pvsc_lattice* lat, int prec, int feat, Sweep& p, cudaStream_t st);
 int launch_sweep_shape(const pvsc_lattice* lat, int prec, int feat, Sweep& p, LaunchShape sh, cudaStream_t st);
 // Link sweep k of a chain of KPM sweeps (consecutive k, the same Sweep p, `partials` the rows of a
-// work buffer) to the one before: each sweep but the last leaves the rows of its dot products,
-// in one of two buffers in turn, to the next one.  Call kpm_chain before the launch of a sweep and
-// kpm_launched after it.
-void kpm_chain(const pvsc_lattice* lat, Sweep& p, double* partials, int k, bool last);
+// work buffer) to the one before: each sweep leaves the rows of its dot products, in one of two
+// buffers in turn, to the next one.  Call kpm_chain before the launch of a sweep and kpm_launched
+// after it; the rows of the last are summed by launch_sum_rows.
+void kpm_chain(const pvsc_lattice* lat, Sweep& p, double* partials, int k);
 void kpm_launched(Sweep& p);
+int launch_sum_rows(const Sweep& p, cudaStream_t st);  // outputs of the rows that p's launch wrote
 void set_products(const pvsc_lattice* lat, int prec, Sweep& p);  // Sweep::pd or pf from coef
 int kpm_enqueue(const pvsc_lattice* lat, int R, int prec, const void* r0, uint64_t seed, int M, double a,
                 double b, double* mu, void* work, const LaunchShape* force, cudaStream_t cs);

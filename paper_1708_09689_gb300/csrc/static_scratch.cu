@@ -2,8 +2,7 @@
 // allocate device memory.
 //
 // pvsc_cheb_step needs a caller-provided work buffer for the per-block dot
-// product partials and the arrival counter of its last-block reduction.  Some
-// callers have no way to provide one: code that runs after start-up under a
+// product partials.  Some callers have no way to provide one: code that runs after start-up under a
 // fixed device-memory budget (a framework whose pool already owns the free
 // memory), callbacks and plugins that must not call cudaMalloc because it can
 // synchronise the whole device, and hosts that forbid allocation once they are
@@ -17,10 +16,8 @@
 // cheap host call once the module is loaded; nothing is cached, so the address
 // stays right after cudaDeviceReset reloads the module).  The first call on a
 // device loads the module there: make it before any stream capture.  Every
-// call on a device shares the one array and it keeps
-// the contents the previous call left; the arrival counter at its start is
-// cleared (cudaMemsetAsync on the caller's stream) before each sweep.  Calls
-// whose kernels overlap on the GPU (different streams, no ordering) race on
+// call on a device shares the one array; no call reads what an earlier one left
+// there.  Calls whose kernels overlap on the GPU (different streams, no ordering) race on
 // the array: order them on one stream or synchronise between them.
 #include "internal.h"
 

@@ -259,6 +259,7 @@ __global__ void __launch_bounds__(MAXT) ti_kpm2_sweep(const __grid_constant__ Sw
 #pragma unroll
     for (int v = 0; v < VPT; ++v) acc[k][v] = dsum[(k * 2 + v) * nthr + t];
   reduce_dots<VPT, MAXT / 32>(p, acc);
+  finish_dots(p);
 }
 
 // default tile per number of vector chunks C = R / 2: about 380 threads or

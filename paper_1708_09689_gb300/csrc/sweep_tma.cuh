@@ -791,8 +791,8 @@ __global__ void __launch_bounds__(32 * NW, 1)
   __syncthreads();
   if constexpr (has_dots(FEAT)) {
     // fixed-order reduction: the warps' partials in index order, then the
-    // blocks in finish_dots (after an abort the values are garbage, but the
-    // arrival counter stays consistent)
+    // blocks' rows by the next sweep of a chain or launch_sum_rows (after an abort
+    // the values are garbage)
     const double* wd = reinterpret_cast<const double*>(base + L::DOT_OFF);
     constexpr int RV = (FX || CD) ? R / 2 : R;  // vectors of a slice
     constexpr int RVF = RV * SL;        // of the block (this block writes its slice's)
@@ -810,7 +810,6 @@ __global__ void __launch_bounds__(32 * NW, 1)
       }
       row[d * RVF + sl * RV + r] = sum;
     }
-    finish_dots(p, reinterpret_cast<double*>(base));  // the rings are drained
   }
 }
 
