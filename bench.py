@@ -633,10 +633,10 @@ def run_workload(args, pv, dev, rank, world):
                                             "W=1, 16 random-phase vectors, 2048 moments", "launch": lat.get_tuning(R, pv.C64)},
                      "dos_at_E0_per_site": float(pv.dos(lat, mu, E0, a, b)[0].item()) / lat.n_sites,
                      "roofline": _hbm_roof(48.0 + 4.0 / R, lups, ms,
-                                           {7: "ti_sweep_tma<*,*,8,F_DOTS,3> (TMA-staged Weyl cells)",
-                                            0: "wsm_march_sweep<float,2,F_DOTS> (z-marching cells)"}.get(
+                                           {7: "ti_sweep_tma<*,*,8,F_KPM,3> (TMA-staged Weyl cells)",
+                                            0: "wsm_march_sweep<float,2,F_KPM> (z-marching cells)"}.get(
                                                int(lat.get_tuning(R, pv.C64).get("kernel", 1)),
-                                               "wsm_sweep<float,2,F_DOTS> (flat two-site cells)")),
+                                               "wsm_sweep<float,2,F_KPM> (flat two-site cells)")),
                      "clocks": clk, "gpu_launches": args.steps * (M // 2)})
     elif args.workload == "batched":
         specs = W.batched_lattices()
@@ -689,7 +689,7 @@ def run_workload(args, pv, dev, rank, world):
                           "frac": roof_p["frac"], "launch": lats[0].get_tuning(R, pv.C64)}
             lats[0].set_tuning(R, pv.C64, **{k: v for k, v in tuning.items() if k != "time_ms"})
             del work_p
-        mode = ("every lattice's KPM as a chain of TMA-staged sweeps, the chains on 4 forked streams "
+        mode = ("every lattice's KPM as a chain of TMA-staged sweeps, the chains on sixteen forked streams "
                 "in one CUDA graph" if per_lattice else "one persistent cooperative launch in a CUDA graph")
         line.update({"workload": "batched", "value": round(world * lups / (ms * 1e-3) / 1e9, 3),
                      "ms_per_step": round(ms, 3), "steps": args.steps, "dtype": "c64",
@@ -697,7 +697,7 @@ def run_workload(args, pv, dev, rank, world):
                                             "1024 moments, " + mode,
                                 "sites": sites, "mu0_min": float(mu[:, :, 0].min().item()), "launch": tuning},
                      "roofline": _hbm_roof(96.0 + 8.0 / R, lups, ms,
-                                           "ti_sweep_tma<16,F_DOTS> (per-lattice chains)" if per_lattice
+                                           "ti_sweep_tma<16,F_KPM> (per-lattice chains)" if per_lattice
                                            else "kpm_batched_kernel<float,2>"),
                      "clocks": clk, "persistent_launch": persistent,
                      "gpu_launches": args.steps * (len(specs) * (2 + M // 2) if per_lattice else 1)})
@@ -850,19 +850,19 @@ def main():
     elif bool(tuning) and tuning.get("kernel") == 7:
         bytes_per_lup = 96.0 + 4.0 / R
         launches = sweeps
-        kname = f"ti_sweep_tma<{R},F_DOTS> (complex64 KPM sweep, TMA-staged plane tiles)"
+        kname = f"ti_sweep_tma<{R},F_KPM> (complex64 KPM sweep, TMA-staged plane tiles)"
     elif bool(tuning) and tuning.get("kernel") == 8:
         bytes_per_lup = 96.0 + 4.0 / R
         launches = sweeps
-        kname = f"ti_sweep_tma_xm<{R},F_DOTS> (complex64 KPM sweep, TMA-staged tiles marching along x)"
+        kname = f"ti_sweep_tma_xm<{R},F_KPM> (complex64 KPM sweep, TMA-staged tiles marching along x)"
     elif bool(tuning) and tuning.get("kernel") == 6:
         bytes_per_lup = 96.0 + 4.0 / R
         launches = sweeps
-        kname = f"ti_sweep_xmarch<float,{tuning.get('vpt') or 2},F_DOTS> (complex64 KPM sweep marching along x)"
+        kname = f"ti_sweep_xmarch<float,{tuning.get('vpt') or 2},F_KPM> (complex64 KPM sweep marching along x)"
     else:
         bytes_per_lup = 96.0 + 4.0 / R      # x 32 + y_in 32 + y_out 32 (B), fp32 V 4 per site
         launches = sweeps
-        kname = "ti_sweep<float,2,F_DOTS> (complex64 KPM sweep)"
+        kname = "ti_sweep<float,2,F_KPM> (complex64 KPM sweep)"
     launch_ms = ms / launches                # upper bound: includes launch gaps of the graph
     achieved = bytes_per_lup * lups_per_step / (ms * 1e-3) / 1e9
     peak, peak_kind = measured_peaks()

@@ -1,7 +1,7 @@
 // TI sweep with tensor-memory-accelerator (TMA) staging of z-plane tiles
 // (tuning kernel 7; kernel 8 marches the same tiles along x), complex64
-// storage, R = 1 .. 64; the same kernel carries the Weyl-semimetal cells and
-// the fixed-point (PVSC_Q64) KPM sweep.
+// storage, R = 1 .. 64; the same kernel carries the Weyl-semimetal cells, the
+// fixed-point (PVSC_Q64) KPM sweep and the complex128 TI sweep.
 //
 // The stencil of Eq. TB_H_topi reads every x element of a plane seven times
 // (the site itself and its six neighbours).  Here a block owns a tile of
