@@ -1,10 +1,8 @@
 // complex128 storage, fp64 arithmetic: kernel instantiations and launchers
 // (register-marching, flat, cp.async-prefetching and shared-memory staged TI
 // sweeps; graphene sweep).
-#include <mutex>
-#include <set>
-
 #include "internal.h"
+#include "per_device.h"
 #include "sweep.cuh"
 #include "sweep_bulk.cuh"
 
@@ -57,21 +55,20 @@ static void* pick(int model, int feat) {
   }
 }
 
-// Opt a kernel into the device's full dynamic shared memory (once per kernel).
+// Opt a kernel into the current device's full dynamic shared memory (once per kernel and device).
 int allow_max_smem(void* fn) {
-  static std::mutex mu;
-  static std::set<void*> done;
-  std::lock_guard<std::mutex> lk(mu);
-  if (done.count(fn)) return PVSC_OK;
-  int dev = 0, optin = 0;
+  static OncePerDevice<void*> opted;
+  int dev = 0;
   PVSC_CUDA_TRY(cudaGetDevice(&dev));
-  PVSC_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  cudaFuncAttributes fa;
-  PVSC_CUDA_TRY(cudaFuncGetAttributes(&fa, fn));
-  PVSC_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     optin - (int)fa.sharedSizeBytes));
-  done.insert(fn);
-  return PVSC_OK;
+  return opted.run(dev, fn, [&]() -> int {
+    int optin = 0;
+    PVSC_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    cudaFuncAttributes fa;
+    PVSC_CUDA_TRY(cudaFuncGetAttributes(&fa, fn));
+    PVSC_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       optin - (int)fa.sharedSizeBytes));
+    return PVSC_OK;
+  });
 }
 
 int launch_sweep_c128(int model, int feat, int grid, int threads, const Sweep& p,
