@@ -21,6 +21,7 @@
 // order by every block).
 #include <cmath>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <type_traits>
 #include <vector>
@@ -28,6 +29,7 @@
 #include <algorithm>
 
 #include "internal.h"
+#include "per_device.h"
 #include "sweep.cuh"
 
 namespace pvsc {
@@ -300,6 +302,29 @@ static BatchShape batch_shape(const pvsc_lattice* l0, int R, int prec) {
 // 62.0, 65.5 and 63.6 GLUP/s on 4, 8, 16 and 32.
 constexpr int kBatchStreams = 16;
 
+// The streams of one device, and the events that fork them from and join them to a caller's stream;
+// calls from several host threads take turns on them.
+struct BatchStreams {
+  cudaStream_t stream[kBatchStreams] = {};
+  cudaEvent_t fork = nullptr, join[kBatchStreams] = {};
+  std::unique_ptr<std::mutex> mu;
+};
+
+static int batch_streams(BatchStreams** out) {
+  static PerDevice<BatchStreams> pools;
+  int dev = 0;
+  PVSC_CUDA_TRY(cudaGetDevice(&dev));
+  return pools.get(dev, out, [](BatchStreams& b) -> int {
+    for (int k = 0; k < kBatchStreams; ++k) {
+      PVSC_CUDA_TRY(cudaStreamCreateWithFlags(&b.stream[k], cudaStreamNonBlocking));
+      PVSC_CUDA_TRY(cudaEventCreateWithFlags(&b.join[k], cudaEventDisableTiming));
+    }
+    PVSC_CUDA_TRY(cudaEventCreateWithFlags(&b.fork, cudaEventDisableTiming));
+    b.mu = std::make_unique<std::mutex>();
+    return PVSC_OK;
+  });
+}
+
 static bool per_lattice_possible(const pvsc_lattice* const* lats, int n, int R, int prec) {
   for (int i = 0; i < n; ++i)
     if (!lats[i] || !tma_sweep_possible(lats[i], R, prec)) return false;
@@ -338,19 +363,9 @@ static int kpm_per_lattice(const pvsc_lattice* const* lats, int n, int R, int pr
   const size_t total = chains_bytes(lats, n, R, prec);
   for (int i = 1; i < n; ++i) off[i] = off[i - 1] + ((per_lattice_bytes(lats[i - 1], R, prec) + 255) & ~size_t(255));
   if (work_bytes < total) return set_error(PVSC_ERR_ARG, "work buffer too small: %zu < %zu", work_bytes, total);
-  static std::mutex mu_streams;
-  static cudaStream_t pool[kBatchStreams];
-  static cudaEvent_t fork_ev, join_ev[kBatchStreams];
-  static bool ready = false;
-  std::lock_guard<std::mutex> lk(mu_streams);
-  if (!ready) {
-    for (int k = 0; k < kBatchStreams; ++k) {
-      PVSC_CUDA_TRY(cudaStreamCreateWithFlags(&pool[k], cudaStreamNonBlocking));
-      PVSC_CUDA_TRY(cudaEventCreateWithFlags(&join_ev[k], cudaEventDisableTiming));
-    }
-    PVSC_CUDA_TRY(cudaEventCreateWithFlags(&fork_ev, cudaEventDisableTiming));
-    ready = true;
-  }
+  BatchStreams* bp = nullptr;
+  if (int rc = batch_streams(&bp)) return rc;
+  std::lock_guard<std::mutex> lk(*bp->mu);
   // the largest lattices first, each on the stream with the least work so far
   std::vector<int> order(n);
   for (int i = 0; i < n; ++i) order[i] = i;
@@ -382,8 +397,8 @@ static int kpm_per_lattice(const pvsc_lattice* const* lats, int n, int R, int pr
     uid.insert(uid.end(), {(uint64_t)(uintptr_t)lats[i], lats[i]->generation, seeds[i], ab[0], ab[1]});
   }
   auto body = [&](cudaStream_t cs) -> int {
-    PVSC_CUDA_TRY(cudaEventRecord(fork_ev, cs));
-    for (int k = 0; k < kBatchStreams; ++k) PVSC_CUDA_TRY(cudaStreamWaitEvent(pool[k], fork_ev, 0));
+    PVSC_CUDA_TRY(cudaEventRecord(bp->fork, cs));
+    for (int k = 0; k < kBatchStreams; ++k) PVSC_CUDA_TRY(cudaStreamWaitEvent(bp->stream[k], bp->fork, 0));
     double load[kBatchStreams] = {};
     for (int i : order) {
       int k = 0;
@@ -396,12 +411,12 @@ static int kpm_per_lattice(const pvsc_lattice* const* lats, int n, int R, int pr
         sh.zslab = (int)std::min<double>(std::max(depth, 1.0), (double)lats[i]->g.L[2]);
       }
       if (int rc = kpm_enqueue(lats[i], R, prec, nullptr, seeds[i], M, a[i], b[i], mu + (size_t)i * R * M,
-                               static_cast<char*>(work) + off[i], &sh, pool[k]))
+                               static_cast<char*>(work) + off[i], &sh, bp->stream[k]))
         return rc;
     }
     for (int k = 0; k < kBatchStreams; ++k) {
-      PVSC_CUDA_TRY(cudaEventRecord(join_ev[k], pool[k]));
-      PVSC_CUDA_TRY(cudaStreamWaitEvent(cs, join_ev[k], 0));
+      PVSC_CUDA_TRY(cudaEventRecord(bp->join[k], bp->stream[k]));
+      PVSC_CUDA_TRY(cudaStreamWaitEvent(cs, bp->join[k], 0));
     }
     return PVSC_OK;
   };

@@ -28,4 +28,27 @@ class OncePerDevice {
   std::set<std::pair<int, Key>> done_;
 };
 
+// A T per device: get(device, &t, create) makes it with create(T&) on the first call for that device
+// (kept only if that returns 0) and hands out the one of the device.  A T stays where it is.
+template <class T>
+class PerDevice {
+ public:
+  template <class F>
+  int get(int device, T** out, F&& create) {
+    std::lock_guard<std::mutex> lk(mu_);
+    auto it = at_.find(device);
+    if (it == at_.end()) {
+      T t{};
+      if (const int rc = create(t)) return rc;
+      it = at_.emplace(device, std::move(t)).first;
+    }
+    *out = &it->second;
+    return 0;
+  }
+
+ private:
+  std::mutex mu_;
+  std::map<int, T> at_;
+};
+
 }  // namespace pvsc

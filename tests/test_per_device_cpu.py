@@ -39,3 +39,23 @@ def test_a_kernel_attribute_is_set_once_per_device(tmp_path):
   rc = 0;
   CHECK(once.run(2, 7, set) == 0 && calls == 5);
 """)
+
+
+def test_every_device_has_its_own_streams(tmp_path):
+    _run(tmp_path, """
+  struct Pool { int device = -1; };
+  PerDevice<Pool> pools;
+  int made = 0, rc = 0, dev = 0;
+  auto make = [&](Pool& p) { ++made; p.device = dev; return rc; };
+  Pool *a = nullptr, *b = nullptr, *c = nullptr;
+  CHECK(pools.get(0, &a, make) == 0 && a->device == 0 && made == 1);
+  dev = 1;
+  CHECK(pools.get(1, &b, make) == 0 && b->device == 1 && made == 2 && a != b);
+  CHECK(pools.get(0, &c, make) == 0 && c == a && made == 2);
+  rc = -5;
+  dev = 2;
+  CHECK(pools.get(2, &c, make) == -5 && made == 3);  // nothing kept of a failure
+  rc = 0;
+  CHECK(pools.get(2, &c, make) == 0 && made == 4 && c->device == 2);
+  CHECK(a->device == 0 && b->device == 1);
+""")
