@@ -404,7 +404,7 @@ size_t pvsc_propagate_adjoint_work_bytes(const pvsc_lattice* lat, int R, int eve
 
 /*
  * Batched KPM: n independent TI lattices (uneven sizes allowed) x R
- * random-phase vectors each, M moments, in one persistent cooperative launch
+ * random-phase vectors each, M moments, in one call: one persistent cooperative launch
  * that walks a device work list of (lattice, z-slab) units; a unit of step k
  * starts once every unit of its lattice has finished step k-1 (a per-lattice
  * phase counter, bounded spin waits), so the lattices advance independently.
@@ -418,12 +418,15 @@ size_t pvsc_propagate_adjoint_work_bytes(const pvsc_lattice* lat, int R, int eve
  * lattice's KPM instead as its own chain of TMA-staged sweeps (threads 256 or
  * 512: the large tile on 8 or 16 warps), the chains on a few streams forked
  * from `stream` inside one captured graph, the same moments as
- * pvsc_kpm_moments with that kernel and seed; that mode does not synchronise
- * and reports copy-wait timeouts through pvsc_device_error.
+ * pvsc_kpm_moments with that kernel and seed; a call with such an entry does
+ * not synchronise and reports copy-wait timeouts through pvsc_device_error.
+ * Every other call, in either form, waits for `stream` (which may not be
+ * under capture).
  * a, b: HOST arrays of n doubles.  Start vectors: counter hash, stream 1,
  * seed seeds[i] (HOST array of n).  mu: device [n][R][M] doubles.
- * Returns PVSC_ERR_TIMEOUT if a wait exceeded pvsc_set_wait_limit (the
- * kernel then stops cleanly; mu is undefined).
+ * Returns PVSC_ERR_TIMEOUT if a wait of the persistent launch exceeded
+ * pvsc_set_wait_limit or a copy wait of an untuned chain's sweep ran out (the
+ * kernels then stop cleanly; mu is undefined).
  * work: pvsc_batched_work_bytes (it depends on the launch shape: query it
  * after any pvsc_set_tuning on lats[0]).
  */
@@ -520,8 +523,10 @@ int pvsc_set_wait_limit(uint64_t spins);
 /* Fault injection for tests of the bounded waits: while enabled, the first
  * dependency wait of every block in pvsc_kpm_moments_batched targets a phase
  * that is never published, so it runs out after the wait limit and the call
- * returns PVSC_ERR_TIMEOUT with the device context intact.  Host-side switch;
- * nothing faults, traps or hangs.  Off by default. */
+ * returns PVSC_ERR_TIMEOUT with the device context intact; an untuned batch
+ * that runs as chains finds its error word set once the chains are done, as by
+ * a sweep whose copy wait ran out.  Host-side switch; nothing faults, traps or
+ * hangs.  Off by default. */
 int pvsc_debug_inject_stall(int enable);
 
 /*

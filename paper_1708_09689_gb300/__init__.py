@@ -574,7 +574,8 @@ def chebfd(lat: Lattice, lo: float, hi: float, a: float, b: float, n_search: int
 
 
 def kpm_moments_batched(lats, M, a, b, R=16, prec=C64, seeds=None, work=None, mu=None, stream=None):
-    """Batched KPM over several TI lattices in one persistent launch: mu (n, R, M)."""
+    """Batched KPM over several TI lattices in one call: mu (n, R, M).  Waits for the stream, except with
+    a kernel 7 entry on lats[0]; a wait on the device that ran out raises PVSC_ERR_TIMEOUT."""
     n = len(lats)
     hs = (ctypes.c_void_p * n)(*[l.handle.value for l in lats])
     seeds = list(seeds) if seeds is not None else list(range(n))
@@ -637,7 +638,8 @@ def set_wait_limit(spins: int):
 
 
 def inject_stall(enable: bool):
-    """Fault injection: make the batched kernel's first wait target an unpublished phase."""
+    """Fault injection: make the persistent batched kernel's first wait target an unpublished phase, and
+    leave an untuned chain's error word set as by a sweep whose copy wait ran out."""
     _check(_lib.pvsc_debug_inject_stall(int(bool(enable))))
 
 

@@ -20,6 +20,7 @@
 // for work that some running block will do (units are processed in phase
 // order by every block).
 #include <cmath>
+#include <cstdio>
 #include <cstring>
 #include <memory>
 #include <mutex>
@@ -356,9 +357,11 @@ static bool chains_default(const pvsc_lattice* const* lats, int n, int R, int pr
   return work >= (int64_t)n << 18;
 }
 
+// err (may be null): set to 1 by a sweep whose copy wait ran out, else 0 once the chains are done;
+// it lies in a work header, which these sweeps leave alone.
 static int kpm_per_lattice(const pvsc_lattice* const* lats, int n, int R, int prec, const uint64_t* seeds, int M,
                            const double* a, const double* b, double* mu, void* work, size_t work_bytes,
-                           const BatchShape& bs, cudaStream_t st) {
+                           const BatchShape& bs, int* err, cudaStream_t st) {
   std::vector<size_t> off(n);
   const size_t total = chains_bytes(lats, n, R, prec);
   for (int i = 1; i < n; ++i) off[i] = off[i - 1] + ((per_lattice_bytes(lats[i - 1], R, prec) + 255) & ~size_t(255));
@@ -387,6 +390,7 @@ static int kpm_per_lattice(const pvsc_lattice* const* lats, int n, int R, int pr
   force.tuned = bs.tuned;
   force.kernel = bs.tuned ? kKernelTma : 0;
   force.threads = bs.threads;
+  force.err = err;
   std::vector<uint64_t> uid = {6, (uint64_t)n, (uint64_t)R, (uint64_t)prec, (uint64_t)M,
                                (uint64_t)(uintptr_t)mu, (uint64_t)(uintptr_t)work, (uint64_t)bs.threads,
                                (uint64_t)bs.tuned};
@@ -397,6 +401,7 @@ static int kpm_per_lattice(const pvsc_lattice* const* lats, int n, int R, int pr
     uid.insert(uid.end(), {(uint64_t)(uintptr_t)lats[i], lats[i]->generation, seeds[i], ab[0], ab[1]});
   }
   auto body = [&](cudaStream_t cs) -> int {
+    if (err) PVSC_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), cs));
     PVSC_CUDA_TRY(cudaEventRecord(bp->fork, cs));
     for (int k = 0; k < kBatchStreams; ++k) PVSC_CUDA_TRY(cudaStreamWaitEvent(bp->stream[k], bp->fork, 0));
     double load[kBatchStreams] = {};
@@ -421,6 +426,14 @@ static int kpm_per_lattice(const pvsc_lattice* const* lats, int n, int R, int pr
     return PVSC_OK;
   };
   return run_graph(lats[0], uid, st, body);
+}
+
+// A batched call without a kernel 7 entry ends here: wait for the stream, read the error word.
+static int wait_for_moments(const int* err, const char* what, cudaStream_t st) {
+  int herr = 0;
+  PVSC_CUDA_TRY(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  PVSC_CUDA_TRY(cudaStreamSynchronize(st));
+  return herr ? set_error(PVSC_ERR_TIMEOUT, "%s", what) : PVSC_OK;
 }
 
 static int batched_layout(const pvsc_lattice* const* lats, int n, int R, int prec, int M,
@@ -500,14 +513,22 @@ int pvsc_kpm_moments_batched(const pvsc_lattice* const* lats, int n, int R, int 
     for (int i = 0; i < n; ++i)
       if (lats[i]->g.model != PVSC_TI || lats[i]->g.zhalo)
         return set_error(PVSC_ERR_UNSUPPORTED, "batched KPM takes TI lattices without halo planes");
-    return kpm_per_lattice(lats, n, R, prec, seeds, M, a, b, mu, work, work_bytes, sh,
+    return kpm_per_lattice(lats, n, R, prec, seeds, M, a, b, mu, work, work_bytes, sh, nullptr,
                            static_cast<cudaStream_t>(stream));
   }
-  // (an injected stall is one of the persistent launch's waits; a work buffer that holds only
-  // the persistent launch gets it)
-  if (!g_inject_stall && chains_default(lats, n, R, prec, sh) && work_bytes >= chains_bytes(lats, n, R, prec))
-    return kpm_per_lattice(lats, n, R, prec, seeds, M, a, b, mu, work, work_bytes, sh,
-                           static_cast<cudaStream_t>(stream));
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  // (a work buffer that holds only the persistent launch gets it)
+  if (chains_default(lats, n, R, prec, sh) && work_bytes >= chains_bytes(lats, n, R, prec)) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    PVSC_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
+    if (cap != cudaStreamCaptureStatusNone)
+      return set_error(PVSC_ERR_CUDA, "a batch without a kernel 7 entry waits for its stream, which is being captured");
+    int* err = static_cast<int*>(work);
+    if (int rc = kpm_per_lattice(lats, n, R, prec, seeds, M, a, b, mu, work, work_bytes, sh, err, st)) return rc;
+    // an injected stall: the mark that a sweep leaves whose wait ran out
+    if (g_inject_stall) PVSC_CUDA_TRY(cudaMemsetAsync(err, 1, sizeof(int), st));
+    return wait_for_moments(err, "a copy wait of a batched-KPM sweep ran out", st);
+  }
   const int threads = sh.threads;
   std::vector<BatchLat> L;
   size_t total = 0;
@@ -558,7 +579,6 @@ int pvsc_kpm_moments_batched(const pvsc_lattice* const* lats, int n, int R, int 
   args.err = err;
   args.wait_limit = g_wait_limit;
   args.inject_stall = g_inject_stall;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
   std::vector<uint64_t> key = {5, (uint64_t)n, (uint64_t)R, (uint64_t)prec, (uint64_t)M,
                                (uint64_t)(uintptr_t)mu, (uint64_t)(uintptr_t)work, g_wait_limit,
                                (uint64_t)grid, (uint64_t)g_inject_stall};
@@ -575,11 +595,9 @@ int pvsc_kpm_moments_batched(const pvsc_lattice* const* lats, int n, int R, int 
     return PVSC_OK;
   };
   if (int rc = run_graph(lats[0], key, st, body)) return rc;
-  int herr = 0;
-  PVSC_CUDA_TRY(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
-  PVSC_CUDA_TRY(cudaStreamSynchronize(st));
-  if (herr) return set_error(PVSC_ERR_TIMEOUT, "a batched-KPM wait exceeded %llu spins", g_wait_limit);
-  return PVSC_OK;
+  char what[96];
+  std::snprintf(what, sizeof(what), "a batched-KPM wait exceeded %llu spins", (unsigned long long)args.wait_limit);
+  return wait_for_moments(err, what, st);
 }
 
 // Launch-shape autotuner of the batched KPM over the whole batch: threads per

@@ -281,6 +281,7 @@ struct Sweep {
   long long fx_kt;       // -alpha t / 2 in Q3.60
   int fx_dshift;         // 1: alpha = 2/a (d doubled)
   const double* vscale;  // per vector: value of one unit of a dot product
+  int* err;              // set to 1 by a block whose copy wait ran out (may be null: the device word alone)
   int zslab;             // TI z-marching depth
   int tile_x, tile_y;    // TI shared-memory staged sweep: tile of columns (0: register marching)
   QDScal qds;            // graphene quantum-dot array (g.v_mode 3): range-test scalars

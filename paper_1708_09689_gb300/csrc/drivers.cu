@@ -537,6 +537,7 @@ int kpm_enqueue(const pvsc_lattice* lat, int R, int prec, const void* r0, uint64
   p.yin = nullptr;
   p.yout = wb;
   p.dot_mode = 1;
+  p.err = sh.err;
   // two steps per sweep: four dots a row and no chain
   if (!two) kpm_chain(lat, p, rows, 0);
   if (int rc = launch_sweep_shape(lat, prec, F_KPM, p, sh, cs)) return rc;

@@ -42,6 +42,7 @@ struct LaunchShape {
                           // 7 TMA-staged plane tiles (warp-specialised)
   bool side_by_side = false;  // one of several sweeps that run at once: zslab holds for an untuned sweep too
   bool tuned = false;     // the fields above are a tuning entry's; else the library's own choice
+  int* err = nullptr;     // Sweep::err of the sweeps of kpm_enqueue
 };
 
 // kernel-selector "model" values of the flat and the cp.async-prefetching TI

@@ -790,6 +790,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
   }
   __syncthreads();
   if constexpr (has_dots(FEAT)) {
+    if (threadIdx.x == 0 && s_abort && p.err != nullptr) atomicExch(p.err, 1);
     // fixed-order reduction: the warps' partials in index order, then the
     // blocks' rows by the next sweep of a chain or launch_sum_rows (after an abort
     // the values are garbage)
