@@ -637,6 +637,9 @@ int pvsc_debug_neighbours(const pvsc_lattice* lat, int64_t* nbr_dev, void* strea
  * first.  D at most 2^24 (PVSC_ERR_ARG otherwise). */
 int pvsc_debug_export_pattern(const pvsc_lattice* lat, int64_t* rowptr, int32_t* col);
 
+/* The captured graphs that the handle keeps and their nodes in all (debug). */
+int pvsc_debug_graph_cache(const pvsc_lattice* lat, int* graphs, int64_t* nodes);
+
 /* Fixed-point arithmetic of the PVSC_Q64 sweeps (debug/parity): runs the
  * device routines those sweeps use on caller-given 64-bit integers, so that
  * they can be checked against exact integer arithmetic.

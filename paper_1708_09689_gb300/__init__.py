@@ -117,6 +117,7 @@ _SIGNATURES = {
     "pvsc_autotune": (_i, [_vp, _i, _i, ctypes.POINTER(Tuning), _vp]),
     "pvsc_autotune_op": (_i, [_vp, _i, _i, _i, ctypes.POINTER(Tuning), _vp]),
     "pvsc_autotune_batched": (_i, [_vp, _i, _i, _i, _vp, _i, _vp, _vp, ctypes.POINTER(Tuning), _vp]),
+    "pvsc_debug_graph_cache": (_i, [_vp, ctypes.POINTER(_i), ctypes.POINTER(ctypes.c_int64)]),
     "pvsc_debug_neighbours": (_i, [_vp, _vp, _vp]),
     "pvsc_last_error": (ctypes.c_char_p, []),
     "pvsc_version": (ctypes.c_char_p, []),
@@ -614,6 +615,13 @@ def debug_series_plan(K: int) -> list:
     out = (ctypes.c_int * max(K, 1))()
     _check(_lib.pvsc_debug_series_plan(K, ctypes.cast(out, ctypes.c_void_p)))
     return list(out)[:K]
+
+
+def debug_graph_cache(lat: Lattice) -> tuple:
+    """(graphs, nodes): the captured graphs that a lattice keeps and their nodes in all."""
+    graphs, nodes = ctypes.c_int(0), ctypes.c_int64(0)
+    _check(_lib.pvsc_debug_graph_cache(lat.handle, ctypes.byref(graphs), ctypes.byref(nodes)))
+    return graphs.value, nodes.value
 
 
 def debug_fx_arith(op: int, values, stream=None):

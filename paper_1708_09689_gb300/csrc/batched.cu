@@ -298,7 +298,8 @@ static BatchShape batch_shape(const pvsc_lattice* l0, int R, int prec) {
 // TMA-staged sweeps (kpm_enqueue), the chains spread over a few streams that
 // fork from and join the caller's stream, all inside one captured graph; a
 // large lattice's sweeps fill the GPU while the small lattices' short sweeps
-// run beside them.  Work: per lattice the dot header and partials and its two
+// run beside them.  With such an entry all of it is one captured graph; an untuned batch
+// captures only what it is called with again (chains_captured).  Work: per lattice the dot header and partials and its two
 // recurrence vectors.  Sixteen streams: the 64-cube benchmark batch ran at 57.7,
 // 62.0, 65.5 and 63.6 GLUP/s on 4, 8, 16 and 32.
 constexpr int kBatchStreams = 16;
@@ -342,11 +343,29 @@ static size_t chains_bytes(const pvsc_lattice* const* lats, int n, int R, int pr
   return total;
 }
 
+// Whether the chains of an untuned batch run as a captured graph: when the same argument set (vectors'
+// seeds, scalings, buffers) was among the last four of the first lattice, and the graph is no larger
+// than the cache holds.  A disorder average has new seeds in every call, and capturing and
+// instantiating a graph costs more than its launches: sixteen cubes of 24 .. 64, R = 16, 64 moments:
+// 13.9 ms enqueued directly, 16.0 captured for one call, 13.6 replayed; of 26, R = 16, 256 moments:
+// 13.8, 21.2 and 12.1; R = 4: 6.1, 7.1 and 4.8.  64 cubes, 1024 moments (33 k nodes): 844, 952 and
+// 810 ms, with 1 GB of host and 0.27 GB of device memory for each graph kept.
+static bool chains_captured(const pvsc_lattice* clat, const std::vector<uint64_t>& key, size_t nodes) {
+  if (nodes > kMaxChainNodes) return false;
+  pvsc_lattice* lat = const_cast<pvsc_lattice*>(clat);
+  std::lock_guard<std::mutex> lk(lat->mu);
+  if (lat->graphs.count(key)) return true;
+  for (const auto& k : lat->batches_seen)
+    if (k == key) return true;
+  lat->batches_seen.push_back(key);
+  if (lat->batches_seen.size() > 4) lat->batches_seen.pop_front();
+  return false;
+}
+
 // Without a tuning entry on the first lattice a complex64 batch runs as chains of untuned sweeps
 // where its lattices hold 2^18 site-vectors on average.  The persistent launch -> chains, 64 moments:
-// sixteen cubes of 24 .. 64, R = 16: 22.7 -> 13.5 ms, R = 4 (413 k site-vectors): 8.1 -> 4.8 ms (6.5
-// with the graph's capture in a first call, 8.3 persistent); of 16 .. 28, R = 16 (176 k): 3.1 -> 2.3 ms,
-// but 3.9 against 3.2 in a first call.
+// sixteen cubes of 24 .. 64, R = 16: 21.5 -> 13.6 ms (13.9 in a first call), R = 4 (413 k site-vectors):
+// 7.8 -> 4.8 ms (6.1 in a first call); of 16 .. 28, R = 16 (176 k): 3.1 -> 2.3 ms replayed.
 static bool chains_default(const pvsc_lattice* const* lats, int n, int R, int prec, const BatchShape& sh) {
   if (sh.tuned || prec != PVSC_C64) return false;
   int64_t work = 0;
@@ -405,6 +424,7 @@ static int kpm_per_lattice(const pvsc_lattice* const* lats, int n, int R, int pr
     PVSC_CUDA_TRY(cudaEventRecord(bp->fork, cs));
     for (int k = 0; k < kBatchStreams; ++k) PVSC_CUDA_TRY(cudaStreamWaitEvent(bp->stream[k], bp->fork, 0));
     double load[kBatchStreams] = {};
+    int rc = PVSC_OK;
     for (int i : order) {
       int k = 0;
       for (int j = 1; j < kBatchStreams; ++j)
@@ -415,17 +435,20 @@ static int kpm_per_lattice(const pvsc_lattice* const* lats, int n, int R, int pr
         sh.side_by_side = true;
         sh.zslab = (int)std::min<double>(std::max(depth, 1.0), (double)lats[i]->g.L[2]);
       }
-      if (int rc = kpm_enqueue(lats[i], R, prec, nullptr, seeds[i], M, a[i], b[i], mu + (size_t)i * R * M,
-                               static_cast<char*>(work) + off[i], &sh, bp->stream[k]))
-        return rc;
+      if ((rc = kpm_enqueue(lats[i], R, prec, nullptr, seeds[i], M, a[i], b[i], mu + (size_t)i * R * M,
+                            static_cast<char*>(work) + off[i], &sh, bp->stream[k])))
+        break;
     }
+    // joined after an error too: what was enqueued uses the caller's buffers
     for (int k = 0; k < kBatchStreams; ++k) {
       PVSC_CUDA_TRY(cudaEventRecord(bp->join[k], bp->stream[k]));
       PVSC_CUDA_TRY(cudaStreamWaitEvent(cs, bp->join[k], 0));
     }
-    return PVSC_OK;
+    return rc;
   };
-  return run_graph(lats[0], uid, st, body);
+  const size_t nodes = (size_t)n * ((M + 1) / 2 + 2);  // start vectors, sweeps, last row sum
+  if (bs.tuned) return run_graph(lats[0], uid, st, body);
+  return chains_captured(lats[0], uid, nodes) ? run_graph(lats[0], uid, st, body, nodes) : body(st);
 }
 
 // A batched call without a kernel 7 entry ends here: wait for the stream, read the error word.
@@ -480,6 +503,21 @@ int pvsc_debug_inject_stall(int enable) {
 int pvsc_set_wait_limit(uint64_t spins) {
   if (spins == 0) return set_error(PVSC_ERR_ARG, "the wait limit must be at least 1");
   g_wait_limit = spins;
+  return PVSC_OK;
+}
+
+int pvsc_debug_graph_cache(const pvsc_lattice* lat, int* graphs, int64_t* nodes) {
+  if (int rc = check_lattice(lat)) return rc;
+  if (!graphs || !nodes) return set_error(PVSC_ERR_ARG, "graphs and nodes must not be NULL");
+  pvsc_lattice* l = const_cast<pvsc_lattice*>(lat);
+  std::lock_guard<std::mutex> lk(l->mu);
+  *graphs = (int)l->graphs.size();
+  *nodes = 0;
+  for (const auto& kv : l->graphs) {
+    size_t n = 0;
+    PVSC_CUDA_TRY(cudaGraphGetNodes(kv.second.graph, nullptr, &n));
+    *nodes += (int64_t)n;
+  }
   return PVSC_OK;
 }
 

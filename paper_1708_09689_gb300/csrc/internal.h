@@ -7,6 +7,7 @@
 #include <atomic>
 #include <cstdlib>
 
+#include <deque>
 #include <map>
 #include <mutex>
 #include <string>
@@ -138,7 +139,8 @@ struct Graph {
 struct pvsc_lattice;
 namespace pvsc {
 template <class F>
-int run_graph(const pvsc_lattice* clat, const std::vector<uint64_t>& key, cudaStream_t st, F&& body);
+int run_graph(const pvsc_lattice* clat, const std::vector<uint64_t>& key, cudaStream_t st, F&& body,
+              size_t nodes = 0);
 }
 
 struct pvsc_lattice {
@@ -156,6 +158,8 @@ struct pvsc_lattice {
   std::map<std::pair<int, int>, pvsc_tuning> tuning;  // (R, prec) -> tuning
   // cached CUDA graphs keyed by the full argument set of a captured loop
   std::map<std::vector<uint64_t>, pvsc::Graph> graphs;
+  size_t graph_nodes = 0;  // kernel nodes of the batches' chains among them (at most kMaxChainNodes)
+  std::deque<std::vector<uint64_t>> batches_seen;  // argument sets of the latest untuned batches
   // Process-unique stamp of the lattice's state, renewed whenever its cached
   // graphs go stale (creation, new potential, new tuning): graphs that capture
   // other lattices' geometry (the batched KPM) key on it, so that a changed
@@ -239,6 +243,8 @@ inline void drop_graphs(pvsc_lattice* lat) {
     if (kv.second.graph) cudaGraphDestroy(kv.second.graph);
   }
   lat->graphs.clear();
+  lat->graph_nodes = 0;
+  lat->batches_seen.clear();
 }
 
 // Programmatic dependent launch of the TMA-staged and the complex128 graphene sweeps (on unless
@@ -253,20 +259,27 @@ inline bool graphs_enabled() {
   return !(e && e[0] && e[0] != '0');
 }
 
+// The chains of untuned batches keep graphs of at most this many kernel nodes in all on a lattice:
+// a node's parameters take about 30 KB of host and 8 KB of device memory once instantiated.
+constexpr size_t kMaxChainNodes = 4096;
+
+// nodes > 0: the kernel nodes of an untuned batch's chains (at most kMaxChainNodes), counted against
+// that bound.
 template <class F>
 int run_graph(const pvsc_lattice* clat, const std::vector<uint64_t>& key, cudaStream_t st,
-                     F&& body) {
+                     F&& body, size_t nodes) {
   if (!graphs_enabled()) return body(st);
   pvsc_lattice* lat = const_cast<pvsc_lattice*>(clat);
   std::lock_guard<std::mutex> lk(lat->mu);
   auto it = lat->graphs.find(key);
   if (it == lat->graphs.end()) {
-    if (lat->graphs.size() >= 32) {
+    if (lat->graphs.size() >= 32 || (nodes > 0 && lat->graph_nodes + nodes > kMaxChainNodes)) {
       for (auto& kv : lat->graphs) {
         cudaGraphExecDestroy(kv.second.exec);
         cudaGraphDestroy(kv.second.graph);
       }
       lat->graphs.clear();
+      lat->graph_nodes = 0;
     }
     cudaStream_t cs;
     PVSC_CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
@@ -287,6 +300,7 @@ int run_graph(const pvsc_lattice* clat, const std::vector<uint64_t>& key, cudaSt
       return body(st);
     }
     it = lat->graphs.emplace(key, gr).first;
+    lat->graph_nodes += nodes;
   }
   PVSC_CUDA_TRY(cudaGraphLaunch(it->second.exec, st));
   return PVSC_OK;
