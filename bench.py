@@ -358,9 +358,8 @@ TI_KERNEL_NAMES = {0: "ti_sweep (z-march)", 1: "ti_sweep_flat", 2: "ti_sweep (cp
                    8: "ti_sweep_tma (TMA-staged tiles marching along x)"}
 
 
-def ti_kernel_name(tuning: dict, what: str) -> str:
-    """The TI sweep a tuning entry selects, for the roofline record."""
-    k = int(tuning.get("kernel", 0)) if tuning else 0
+def ti_kernel_name(k: int, what: str) -> str:
+    """The TI sweep of kernel number k (what the lattice runs, tuned or not), for the roofline record."""
     return f"{TI_KERNEL_NAMES.get(k, 'ti_sweep')} {what}"
 
 
@@ -544,7 +543,7 @@ def run_workload(args, pv, dev, rank, world):
                                 "launch": lat.get_tuning(R, pv.C64)},
                      "density_ms_64k": round(t_d, 4),
                      "peak_at_k0": peak(32, 0.5, 1.5), "closed_form_k0": 1.0,
-                     "roofline": _hbm_roof(96.0, lups, ms, ti_kernel_name(lat.get_tuning(R, pv.C64),
+                     "roofline": _hbm_roof(96.0, lups, ms, ti_kernel_name(pv.debug_route(lat, R, pv.C64),
                                                                          "KPM sweeps (R = 64, V = 0)")),
                      "clocks": clk, "gpu_launches": args.steps * len(calls) * ((M + 1) // 2 + 1 + nk_call)})
     elif args.workload == "chebfd":
@@ -595,7 +594,7 @@ def run_workload(args, pv, dev, rank, world):
                      "max_residual": float(res[inside].max()) if n_in else None,
                      "kramers_pairs": bool(n_in % 2 == 0),
                      "roofline": _hbm_roof(96.0 + 8.0 / ns + 128.0 / 3, lups, 1000 * secs,
-                                           ti_kernel_name(lat.get_tuning(ns, pv.C64),
+                                           ti_kernel_name(pv.debug_route(lat, ns, pv.C64),
                                                           "series sweeps (R = 64; accumulator on every "
                                                           "third sweep), solver average")),
                      "clocks": clk, "gpu_launches": None})
@@ -635,7 +634,7 @@ def run_workload(args, pv, dev, rank, world):
                      "roofline": _hbm_roof(48.0 + 4.0 / R, lups, ms,
                                            {7: "ti_sweep_tma<*,*,8,F_KPM,3> (TMA-staged Weyl cells)",
                                             0: "wsm_march_sweep<float,2,F_KPM> (z-marching cells)"}.get(
-                                               int(lat.get_tuning(R, pv.C64).get("kernel", 1)),
+                                               pv.debug_route(lat, R, pv.C64),
                                                "wsm_sweep<float,2,F_KPM> (flat two-site cells)")),
                      "clocks": clk, "gpu_launches": args.steps * (M // 2)})
     elif args.workload == "batched":
@@ -672,11 +671,12 @@ def run_workload(args, pv, dev, rank, world):
         clk = clocks.stop()
         sites = sum(L ** 3 for L, _, _ in specs)
         lups = sites * R * (M // 2)
-        per_lattice = bool(tuning) and int(tuning.get("kernel", 0)) == 7
+        per_lattice = pv.debug_batched_route(lats, R, pv.C64, work.numel())
         persistent = None
         if per_lattice:
             # the batch as the one persistent cooperative launch too (its measured best shape:
             # 256 threads, one block per SM, whole columns), for the record
+            shape = {k: v for k, v in lats[0].get_tuning(R, pv.C64).items() if k != "time_ms"}
             lats[0].set_tuning(R, pv.C64, threads=256, blocks_per_sm=1, zslab=0, kernel=0)
             work_p = pv.work_buffer(pv.batched_work_bytes(lats, R, pv.C64, M), dev)
             run_p = lambda: pv.kpm_moments_batched(lats, M, [x[0] for x in ab], [x[1] for x in ab], R=R,
@@ -687,10 +687,10 @@ def run_workload(args, pv, dev, rank, world):
             roof_p = _hbm_roof(96.0 + 8.0 / R, lups, ms_p, "kpm_batched_kernel<float,2>")
             persistent = {"value": round(world * lups / (ms_p * 1e-3) / 1e9, 3), "ms_per_step": round(ms_p, 3),
                           "frac": roof_p["frac"], "launch": lats[0].get_tuning(R, pv.C64)}
-            lats[0].set_tuning(R, pv.C64, **{k: v for k, v in tuning.items() if k != "time_ms"})
+            lats[0].set_tuning(R, pv.C64, **shape)
             del work_p
-        mode = ("every lattice's KPM as a chain of TMA-staged sweeps, the chains on sixteen forked streams "
-                "in one CUDA graph" if per_lattice else "one persistent cooperative launch in a CUDA graph")
+        mode = ("every lattice's KPM as a chain of TMA-staged sweeps, the chains on sixteen forked streams"
+                if per_lattice else "one persistent cooperative launch in a CUDA graph")
         line.update({"workload": "batched", "value": round(world * lups / (ms * 1e-3) / 1e9, 3),
                      "ms_per_step": round(ms, 3), "steps": args.steps, "dtype": "c64",
                      "config": {"workload": "64 periodic TI cubes, L from {24,32,48,64,96}, W~U[0,5), R=16, "
@@ -840,25 +840,26 @@ def main():
     mu64 = mu.clone()
 
     # ---- roofline of the dominant kernel (the complex64 TI KPM sweep)
-    two_step = bool(tuning) and tuning.get("kernel") == 4
+    route = pv.debug_route(lat, R, pv.C64)
+    two_step = route == 4
     if two_step:
         # two recurrence steps per launch: w_{k-1}, w_k read and w_{k+1}, w_{k+2} written
         # once (4 x 32 B per site and vector over two steps), the fp32 potential once
         bytes_per_lup = 64.0 + 2.0 / R
         launches = 1 + (sweeps - 1) // 2 + (sweeps - 1) % 2
         kname = "ti_kpm2_sweep (complex64, two KPM steps per sweep)"
-    elif bool(tuning) and tuning.get("kernel") == 7:
+    elif route == 7:
         bytes_per_lup = 96.0 + 4.0 / R
         launches = sweeps
         kname = f"ti_sweep_tma<{R},F_KPM> (complex64 KPM sweep, TMA-staged plane tiles)"
-    elif bool(tuning) and tuning.get("kernel") == 8:
+    elif route == 8:
         bytes_per_lup = 96.0 + 4.0 / R
         launches = sweeps
         kname = f"ti_sweep_tma_xm<{R},F_KPM> (complex64 KPM sweep, TMA-staged tiles marching along x)"
-    elif bool(tuning) and tuning.get("kernel") == 6:
+    elif route == 6:
         bytes_per_lup = 96.0 + 4.0 / R
         launches = sweeps
-        kname = f"ti_sweep_xmarch<float,{tuning.get('vpt') or 2},F_KPM> (complex64 KPM sweep marching along x)"
+        kname = f"ti_sweep_xmarch<float,{lat.get_tuning(R, pv.C64)['vpt'] or 2},F_KPM> (complex64 KPM sweep marching along x)"
     else:
         bytes_per_lup = 96.0 + 4.0 / R      # x 32 + y_in 32 + y_out 32 (B), fp32 V 4 per site
         launches = sweeps

@@ -535,8 +535,13 @@ int pvsc_debug_inject_stall(int enable);
  * depth of the TI z-marching sweep (0 = automatic).  pvsc_autotune times the
  * candidates on the device with CUDA events (synchronous; the vectors it
  * sweeps are allocated inside and freed) and stores the winner in the
- * handle; pvsc_get_tuning reads the entry in force.
+ * handle; pvsc_get_tuning reads the entry in force.  Without one it reads
+ * kernel = PVSC_UNTUNED, the library's own choice per sweep, and so does `best`
+ * of an autotuner whose winner is that choice; given back to pvsc_set_tuning,
+ * such a struct removes the entry (its other fields are not read).
+ * (PVSC_Q64 reads a shape of its own and has no such value.)
  */
+#define PVSC_UNTUNED (-1)
 typedef struct {
   int32_t threads;
   int32_t blocks_per_sm; /* resident blocks per SM (0: from occupancy); kernels 7 and 8: 0 or 1, */
@@ -582,9 +587,10 @@ typedef struct {
                   /* the next sweep's blocks set up on free SMs and wait for the */
                   /* previous sweep to complete before touching global memory (same */
                   /* results; environment PVSC_NO_PDL=1 launches them plainly). */
-                  /* Without an entry, complex64 sweeps of TI and Weyl lattices that fill the */
-                  /* chip run kernel 7's tiles (any Lx), the others the z-march (TI) or a */
-                  /* flat cell sweep (Weyl); pvsc_get_tuning then still reads 256 threads, kernel 0. */
+                  /* Without an entry (PVSC_UNTUNED), complex64 sweeps of TI and Weyl lattices */
+                  /* that fill the chip run kernel 7's tiles (any Lx), complex128 sweeps of large */
+                  /* TI blocks the same tiles for complex128 vectors, the others the z-march */
+                  /* (TI) or a flat cell sweep (Weyl). */
                   /* PVSC_Q64 (KPM on TI lattices) takes kernels 0, 2, 3 (threads a */
                   /* multiple of R, one vector per thread, no tile) and 7 for R = 1 .. 32 */
                   /* (any Lx): the tiles, rings and variants of the complex64 layout */
@@ -636,6 +642,14 @@ int pvsc_debug_neighbours(const pvsc_lattice* lat, int64_t* nbr_dev, void* strea
  * col: HOST array of rowptr[D] int32 column indices, or NULL to size it
  * first.  D at most 2^24 (PVSC_ERR_ARG otherwise). */
 int pvsc_debug_export_pattern(const pvsc_lattice* lat, int64_t* rowptr, int32_t* col);
+
+/* The kernel (as in pvsc_tuning) whose form the recurrence sweeps of (R, prec)
+ * take now, chosen by an entry or by the library; a negative status for bad
+ * arguments.  prec: complex128 or complex64.  Host only (debug). */
+int pvsc_debug_route(const pvsc_lattice* lat, int R, int prec);
+/* 1 if pvsc_kpm_moments_batched with a work buffer of that size runs as chains
+ * of sweeps, 0 if as the persistent launch.  Host only (debug). */
+int pvsc_debug_batched_route(const pvsc_lattice* const* lats, int n, int R, int prec, size_t work_bytes);
 
 /* The captured graphs that the handle keeps and their nodes in all (debug). */
 int pvsc_debug_graph_cache(const pvsc_lattice* lat, int* graphs, int64_t* nodes);

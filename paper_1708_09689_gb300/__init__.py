@@ -29,6 +29,7 @@ C128, C64, Q64 = 0, 1, 2  # Q64: fixed-point vectors, pvsc_kpm_moments on TI onl
 KERNEL_NONE, KERNEL_JACKSON, KERNEL_LORENTZ = 0, 1, 2  # damping kernels of kpm_density
 V_ZERO, V_HOST, V_DEVICE, V_SEED, V_ON_THE_FLY, V_QDOT = 0, 1, 2, 3, 4, 5
 DOT_XX, DOT_XY, DOT_YY = 1, 2, 4
+UNTUNED = -1  # kernel of a tuning without an entry
 OP_APPLY, OP_CHEB_STEP, OP_KPM, OP_SERIES, OP_ADJOINT, OP_KPM_BATCHED = 0, 1, 2, 3, 4, 5
 LATTICE_Z_HALO_LO, LATTICE_Z_HALO_HI = 1, 2  # z-slab lattices: halo plane below / above
 
@@ -117,6 +118,8 @@ _SIGNATURES = {
     "pvsc_autotune": (_i, [_vp, _i, _i, ctypes.POINTER(Tuning), _vp]),
     "pvsc_autotune_op": (_i, [_vp, _i, _i, _i, ctypes.POINTER(Tuning), _vp]),
     "pvsc_autotune_batched": (_i, [_vp, _i, _i, _i, _vp, _i, _vp, _vp, ctypes.POINTER(Tuning), _vp]),
+    "pvsc_debug_route": (_i, [_vp, _i, _i]),
+    "pvsc_debug_batched_route": (_i, [_vp, _i, _i, _i, _sz]),
     "pvsc_debug_graph_cache": (_i, [_vp, ctypes.POINTER(_i), ctypes.POINTER(ctypes.c_int64)]),
     "pvsc_debug_neighbours": (_i, [_vp, _vp, _vp]),
     "pvsc_last_error": (ctypes.c_char_p, []),
@@ -320,6 +323,7 @@ class Lattice:
         _check(_lib.pvsc_set_tuning(self._h, R, prec, ctypes.byref(t)))
 
     def get_tuning(self, R: int, prec: int) -> dict:
+        """The launch shape in force, kernel UNTUNED without an entry (then set_tuning with it removes one)."""
         t = Tuning()
         _check(_lib.pvsc_get_tuning(self._h, R, prec, ctypes.byref(t)))
         return t.as_dict()
@@ -615,6 +619,23 @@ def debug_series_plan(K: int) -> list:
     out = (ctypes.c_int * max(K, 1))()
     _check(_lib.pvsc_debug_series_plan(K, ctypes.cast(out, ctypes.c_void_p)))
     return list(out)[:K]
+
+
+def debug_route(lat: Lattice, R: int, prec: int) -> int:
+    """The kernel number whose form the recurrence sweeps of (R, prec) take now, by an entry or untuned."""
+    k = _lib.pvsc_debug_route(lat.handle, R, prec)
+    if k < 0:
+        _check(k)
+    return k
+
+
+def debug_batched_route(lats, R: int, prec: int, work_bytes: int) -> bool:
+    """Whether a batched call with a work buffer of that size runs as chains of sweeps."""
+    hs = (ctypes.c_void_p * len(lats))(*[l.handle.value for l in lats])
+    k = _lib.pvsc_debug_batched_route(hs, len(lats), R, prec, int(work_bytes))
+    if k < 0:
+        _check(k)
+    return bool(k)
 
 
 def debug_graph_cache(lat: Lattice) -> tuple:

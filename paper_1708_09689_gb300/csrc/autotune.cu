@@ -68,15 +68,17 @@ static void cache_store(const std::string& key, const pvsc_tuning& t) {
 }
 
 // The untuned sweep as a candidate, where no tuning entry can select it (the TMA-staged tiles of a
-// lattice with Lx no multiple of 4, and of complex128 vectors): threads = 0 stands for it in the list and in the cache file,
-// and installing it removes the entry.  The caller is told the defaults that pvsc_get_tuning reads.
+// lattice with Lx no multiple of 4, and of complex128 vectors): kernel = PVSC_UNTUNED with threads = 0
+// stands for it in the list and in the cache file, and installing it removes the entry.  The caller is told
+// what pvsc_get_tuning then reads.
+constexpr pvsc_tuning kUntuned{0, 0, 0, 0.f, 0, 0, 0, PVSC_UNTUNED};
 static bool untuned_is_its_own(const pvsc_lattice* lat, int R, int prec) {
   if (prec == PVSC_C128) return tma_c128_default(lat, R);
   return tma_sweep_default(lat, R, prec) && !tma_sweep_possible(lat, R, prec);
 }
 
 static void install(pvsc_lattice* lat, int R, int prec, const pvsc_tuning& t) {
-  if (t.threads > 0) lat->tuning[{R, prec}] = t;
+  if (t.threads > 0 && t.kernel != PVSC_UNTUNED) lat->tuning[{R, prec}] = t;
   else lat->tuning.erase({R, prec});
 }
 
@@ -84,6 +86,7 @@ static pvsc_tuning reported(pvsc_tuning t, int R, int prec) {
   if (t.threads == 0) {
     t.threads = 256;
     t.vpt = vpt_for(R, prec);
+    t.kernel = PVSC_UNTUNED;
   }
   return t;
 }
@@ -202,7 +205,7 @@ extern "C" int pvsc_autotune_op(pvsc_lattice* lat, int R, int prec, int op, pvsc
   // candidate list: z-marching (all shapes), and for TI the flat, prefetching
   // and shared-memory staged sweeps in a few shapes each
   std::vector<pvsc_tuning> cands;
-  if (untuned_is_its_own(lat, R, prec)) cands.push_back(pvsc_tuning{0, 0, 0, 0.f, 0, 0, 0, 0});
+  if (untuned_is_its_own(lat, R, prec)) cands.push_back(kUntuned);
   for (int vpt : vpt_c) {
     const int C = R / vpt;
     for (int th : {64, 128, 256}) {

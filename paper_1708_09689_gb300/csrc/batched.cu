@@ -521,6 +521,16 @@ int pvsc_debug_graph_cache(const pvsc_lattice* lat, int* graphs, int64_t* nodes)
   return PVSC_OK;
 }
 
+int pvsc_debug_batched_route(const pvsc_lattice* const* lats, int n, int R, int prec, size_t work_bytes) {
+  if (!lats || n < 1 || n > kMaxBatch || !valid_R(R) || (prec != PVSC_C128 && prec != PVSC_C64))
+    return set_error(PVSC_ERR_ARG, "bad lattices, R or precision");
+  for (int i = 0; i < n; ++i)
+    if (!lats[i]) return set_error(PVSC_ERR_ARG, "lattice %d is NULL", i);
+  const BatchShape sh = batch_shape(lats[0], R, prec);
+  if (sh.per_lattice && per_lattice_possible(lats, n, R, prec)) return 1;
+  return chains_default(lats, n, R, prec, sh) && work_bytes >= chains_bytes(lats, n, R, prec) ? 1 : 0;
+}
+
 size_t pvsc_batched_work_bytes(const pvsc_lattice* const* lats, int n, int R, int prec, int M) {
   if (!lats || n < 1 || n > kMaxBatch || !valid_R(R) || (prec != PVSC_C128 && prec != PVSC_C64) || M < 1) return 0;
   std::vector<BatchLat> L;
@@ -677,7 +687,7 @@ int pvsc_autotune_batched(pvsc_lattice* const* lats, int n, int R, int prec, con
   };
   l0->tuning.erase({R, prec});
   if (!per_lattice_possible(lats, n, R, prec) && chains_default(lats, n, R, prec, batch_shape(l0, R, prec)))
-    cands.push_back(pvsc_tuning{0, 0, 0, 0.f, 0, 0, 0, 0});
+    cands.push_back(pvsc_tuning{0, 0, 0, 0.f, 0, 0, 0, PVSC_UNTUNED});
   for (const pvsc_tuning& c : cands) {
     install(c);
     wmax = std::max(wmax, pvsc_batched_work_bytes(lats, n, R, prec, M));
@@ -724,7 +734,10 @@ int pvsc_autotune_batched(pvsc_lattice* const* lats, int n, int R, int prec, con
     return rc;
   }
   install(win);
-  if (win.threads == 0) win.threads = 256;  // as an untuned entry reads
+  if (win.threads == 0) {  // as pvsc_get_tuning then reads
+    win.threads = 256;
+    win.vpt = vpt_for(R, prec);
+  }
   drop_graphs(l0);
   if (best) *best = win;
   return PVSC_OK;

@@ -160,6 +160,11 @@ static int default_threads(const pvsc_lattice* lat, int R, int prec) {
   return narrow ? 128 : 256;
 }
 
+int default_kernel(const pvsc_lattice* lat, int R, int prec) {
+  if (prec == PVSC_C128 ? tma_c128_default(lat, R) : tma_sweep_default(lat, R, prec)) return kKernelTma;
+  return lat->g.model == PVSC_WSM ? 1 : 0;
+}
+
 int launch_sweep(const pvsc_lattice* lat, int prec, int feat, Sweep& p, cudaStream_t st) {
   return launch_sweep_shape(lat, prec, feat, p, shape_for(lat, p.R, prec), st);
 }
@@ -188,9 +193,8 @@ int launch_sweep_shape(const pvsc_lattice* lat, int prec, int feat, Sweep& p, La
     sh = LaunchShape{};
     sh.zslab = zs;
   }
-  if (!sh.tuned && prec == PVSC_C128 && !(feat & F_ADJ) && tma_c128_default(lat, p.R))
-    return launch_sweep_tma_c128(lat, feat, p, st);
-  if (!sh.tuned && !(feat & F_ADJ) && tma_sweep_default(lat, p.R, prec)) {
+  if (!sh.tuned && !(feat & F_ADJ) && default_kernel(lat, p.R, prec) == kKernelTma) {
+    if (prec == PVSC_C128) return launch_sweep_tma_c128(lat, feat, p, st);
     // sixteen warps where the accumulator is read and written (its loads are the longest waits)
     LaunchShape d;
     d.threads = (feat & F_ACC) ? 512 : 256;
@@ -1141,7 +1145,7 @@ int pvsc_set_tuning(pvsc_lattice* lat, int R, int prec, const pvsc_tuning* tunin
     return PVSC_OK;
   }
   if (int rc = check_common(lat, R, prec)) return rc;
-  if (!tuning) {
+  if (!tuning || tuning->kernel == PVSC_UNTUNED) {
     lat->tuning.erase({R, prec});
     drop_graphs(lat);
     return PVSC_OK;
@@ -1238,9 +1242,16 @@ int pvsc_get_tuning(const pvsc_lattice* lat, int R, int prec, pvsc_tuning* tunin
     tuning->vpt = vpt_for(R, prec);
     tuning->tile_x = 0;
     tuning->tile_y = 0;
-    tuning->kernel = 0;
+    tuning->kernel = PVSC_UNTUNED;
   }
   return PVSC_OK;
+}
+
+int pvsc_debug_route(const pvsc_lattice* lat, int R, int prec) {
+  if (int rc = check_common(lat, R, prec)) return rc;
+  auto it = lat->tuning.find({R, prec});
+  if (it == lat->tuning.end()) return default_kernel(lat, R, prec);
+  return lat->g.zhalo || lat->g.model == PVSC_GRAPHENE ? 0 : it->second.kernel;
 }
 
 }  // extern "C"

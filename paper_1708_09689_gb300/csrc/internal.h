@@ -118,6 +118,7 @@ int launch_sweep_tma_fx(const pvsc_lattice* lat, Sweep& p, const LaunchShape& sh
 int tma_error_fx(int clear, int* flag);
 // complex128 TI sweeps on TMA-staged tiles (sweep_tma_c128.cu), the choice of untuned sweeps
 bool tma_c128_default(const pvsc_lattice* lat, int R);
+int default_kernel(const pvsc_lattice* lat, int R, int prec);  // of untuned recurrence sweeps, as pvsc_tuning.kernel
 int launch_sweep_tma_c128(const pvsc_lattice* lat, int feat, Sweep& p, cudaStream_t st);
 int tma_error_c128(int clear, int* flag);
 bool tma_tile_valid(int R, int tile_x, int tile_y);  // (0, 0) or one of the two tiles of this R
