@@ -618,8 +618,9 @@ int pvsc_autotune_op(pvsc_lattice* lat, int R, int prec, int op, pvsc_tuning* be
 /* Launch-shape autotuner of the batched KPM over the whole batch (the batched
  * calls read the (R, prec) tuning entry of lats[0]): threads per block (128,
  * 256), z-segment length of the work units (whole columns, 16 .. 64 planes)
- * and blocks per SM (occupancy maximum, 1) are timed with CUDA events on the
- * batch itself running M moments, and the fastest becomes that entry.
+ * and blocks per SM (occupancy maximum, 1), kernel 7's chains and the untuned
+ * chains are timed with CUDA events on the batch itself running M moments, and
+ * the fastest becomes that entry (the untuned chains: no entry).
  * Allocates and frees its own buffers; synchronises the stream.  Query
  * pvsc_batched_work_bytes again afterwards (it depends on the shape). */
 int pvsc_autotune_batched(pvsc_lattice* const* lats, int n, int R, int prec, const uint64_t* seeds,
@@ -650,6 +651,11 @@ int pvsc_debug_route(const pvsc_lattice* lat, int R, int prec);
 /* 1 if pvsc_kpm_moments_batched with a work buffer of that size runs as chains
  * of sweeps, 0 if as the persistent launch.  Host only (debug). */
 int pvsc_debug_batched_route(const pvsc_lattice* const* lats, int n, int R, int prec, size_t work_bytes);
+
+/* The shapes that pvsc_autotune_op times for an operation: *n of them, the
+ * first max written to out (debug; host only). */
+int pvsc_debug_autotune_candidates(const pvsc_lattice* lat, int R, int prec, int op, pvsc_tuning* out, int max,
+                                   int* n);
 
 /* The captured graphs that the handle keeps and their nodes in all (debug). */
 int pvsc_debug_graph_cache(const pvsc_lattice* lat, int* graphs, int64_t* nodes);

@@ -120,6 +120,7 @@ _SIGNATURES = {
     "pvsc_autotune_batched": (_i, [_vp, _i, _i, _i, _vp, _i, _vp, _vp, ctypes.POINTER(Tuning), _vp]),
     "pvsc_debug_route": (_i, [_vp, _i, _i]),
     "pvsc_debug_batched_route": (_i, [_vp, _i, _i, _i, _sz]),
+    "pvsc_debug_autotune_candidates": (_i, [_vp, _i, _i, _i, ctypes.POINTER(Tuning), _i, ctypes.POINTER(_i)]),
     "pvsc_debug_graph_cache": (_i, [_vp, ctypes.POINTER(_i), ctypes.POINTER(ctypes.c_int64)]),
     "pvsc_debug_neighbours": (_i, [_vp, _vp, _vp]),
     "pvsc_last_error": (ctypes.c_char_p, []),
@@ -636,6 +637,14 @@ def debug_batched_route(lats, R: int, prec: int, work_bytes: int) -> bool:
     if k < 0:
         _check(k)
     return bool(k)
+
+
+def debug_autotune_candidates(lat: Lattice, R: int, prec: int, op: int = OP_KPM) -> list:
+    """The launch shapes that Lattice.autotune times for an operation, as dicts."""
+    n = ctypes.c_int(0)
+    out = (Tuning * 512)()
+    _check(_lib.pvsc_debug_autotune_candidates(lat.handle, R, prec, int(op), out, 512, ctypes.byref(n)))
+    return [t.as_dict() for t in out[:n.value]]
 
 
 def debug_graph_cache(lat: Lattice) -> tuple:

@@ -67,14 +67,16 @@ static void cache_store(const std::string& key, const pvsc_tuning& t) {
   std::fclose(f);
 }
 
-// The untuned sweep as a candidate, where no tuning entry can select it (the TMA-staged tiles of a
-// lattice with Lx no multiple of 4, and of complex128 vectors): kernel = PVSC_UNTUNED with threads = 0
-// stands for it in the list and in the cache file, and installing it removes the entry.  The caller is told
-// what pvsc_get_tuning then reads.
+// The untuned sweeps as a candidate, where no tuning entry can select them: the TMA-staged tiles of a
+// lattice with Lx no multiple of 4 and of complex128 vectors, and the mix of a series (plain sweeps on
+// eight warps, accumulating ones on sixteen; an entry holds one count: a filter of 240x240x6 sites,
+// R = 32, K = 100, 27.5 ms, 28.2 with the best entry).  kernel = PVSC_UNTUNED with threads = 0 stands for them
+// in the list and in the cache file, and installing it removes the entry.  The caller is told what
+// pvsc_get_tuning then reads.
 constexpr pvsc_tuning kUntuned{0, 0, 0, 0.f, 0, 0, 0, PVSC_UNTUNED};
-static bool untuned_is_its_own(const pvsc_lattice* lat, int R, int prec) {
-  if (prec == PVSC_C128) return tma_c128_default(lat, R);
-  return tma_sweep_default(lat, R, prec) && !tma_sweep_possible(lat, R, prec);
+static bool untuned_is_its_own(const pvsc_lattice* lat, int R, int prec, int op) {
+  if (default_kernel(lat, R, prec) != kKernelTma) return false;
+  return prec == PVSC_C128 || op == PVSC_OP_SERIES || !tma_sweep_possible(lat, R, prec);
 }
 
 static void install(pvsc_lattice* lat, int R, int prec, const pvsc_tuning& t) {
@@ -89,6 +91,73 @@ static pvsc_tuning reported(pvsc_tuning t, int R, int prec) {
     t.kernel = PVSC_UNTUNED;
   }
   return t;
+}
+
+// The shapes that are timed: z-marching (all shapes), for TI the flat, prefetching and shared-memory
+// staged sweeps in a few shapes each, the TMA-staged tiles, and the untuned sweeps as above.
+static std::vector<pvsc_tuning> candidates(const pvsc_lattice* lat, int R, int prec, int op) {
+  std::vector<int> vpt_c = {1};
+  if (prec == PVSC_C64 && R >= 2) vpt_c.push_back(2);
+  std::vector<int> zslab_c = {0};
+  const bool march = lat->g.model == PVSC_TI || lat->g.model == PVSC_WSM;  // z-marching sweeps
+  if (march)
+    for (int z : {4, 8, 16, 32, 64})
+      if (z < lat->g.L[2]) zslab_c.push_back(z);
+  const std::vector<int> bps_c = {0, 1, 2};
+  std::vector<pvsc_tuning> cands;
+  if (untuned_is_its_own(lat, R, prec, op)) cands.push_back(kUntuned);
+  for (int vpt : vpt_c) {
+    const int C = R / vpt;
+    for (int th : {64, 128, 256}) {
+      if (th % C != 0 || th < C) continue;
+      for (int bps : bps_c)
+        for (int zs : zslab_c) cands.push_back(pvsc_tuning{th, bps, zs, 0.f, vpt, 0, 0, 0});
+      if (march) cands.push_back(pvsc_tuning{th, 0, 0, 0.f, vpt, 0, 0, 1});  // flat variant
+      if (lat->g.model == PVSC_TI) {
+        // column tiles of this many threads (z-marching, kernel 5)
+        const int tiles5[][2] = {{4, 4}, {8, 4}, {4, 8}, {8, 8}, {16, 4}, {16, 2}, {2, 8}};
+        for (const auto& t : tiles5)
+          if (t[0] * t[1] * C == th) cands.push_back(pvsc_tuning{th, 0, 0, 0.f, vpt, t[0], t[1], 5});
+        // marching along x (lattices with a short z extent)
+        if (lat->g.L[0] > lat->g.L[2]) cands.push_back(pvsc_tuning{th, 0, 0, 0.f, vpt, 0, 0, 6});
+        if (!(prec == PVSC_C64 && vpt == 1 && R > 1)) {
+          for (int zs : {0, 16}) cands.push_back(pvsc_tuning{th, 0, zs, 0.f, vpt, 0, 0, 2});
+          cands.push_back(pvsc_tuning{th, 0, 0, 0.f, vpt, 0, 0, 3});
+        }
+      }
+    }
+  }
+  // TMA-staged plane tiles (kernel 7): z-chunks chosen automatically or a few fixed depths
+  if (tma_sweep_possible(lat, R, prec)) {
+    // the half tiles of the deeper rings (R = 32, 64: slices on the tiles of R = 16)
+    const int deep_y = R == 1 ? 16 : (R == 2 || R == 4) ? 8 : 4, deep_x = R >= 16 ? 8 : (R <= 2 ? 32 : 16);
+    // blocks_per_sm 1: spread the planes over every SM when there are fewer units
+    // than SMs (the same launch otherwise, and with automatic chunks, which spread anyway)
+    for (int zs : {0, 16, 32, 64})
+      if (zs == 0 || zs < lat->g.L[2])
+        for (int spread = 0; spread < (zs == 0 ? 1 : 2); ++spread) {
+          cands.push_back(pvsc_tuning{256, spread, zs, 0.f, 2, 0, 0, kKernelTma});
+          cands.push_back(pvsc_tuning{256, spread, zs, 0.f, 2, deep_x, deep_y, kKernelTma});
+          if (lat->g.model == PVSC_TI)  // the Weyl cells run eight warps only
+            cands.push_back(pvsc_tuning{512, spread, zs, 0.f, 2, 0, 0, kKernelTma});
+        }
+    // the same tiles marching along x, where the z columns are the shorter
+    if (lat->g.L[0] > lat->g.L[2] && tma_xm_possible(lat, R, prec))
+      for (int zs : {0, 32, 64})
+        if (zs == 0 || zs < lat->g.L[0]) {
+          cands.push_back(pvsc_tuning{256, 0, zs, 0.f, 2, 0, 0, kKernelTmaX});
+          if (lat->g.model == PVSC_TI) cands.push_back(pvsc_tuning{256, 0, zs, 0.f, 2, deep_x, deep_y, kKernelTmaX});
+        }
+  }
+  if (lat->g.model == PVSC_TI)
+    for (int th : {128, 256}) {
+      if (th % R) continue;
+      const int tiles[][2] = {{32, 8}, {16, 8}, {16, 4}, {8, 8}, {8, 4}, {4, 4}};
+      for (const auto& t : tiles)
+        if (t[0] * t[1] <= 2 * th && bulk_smem_bytes(t[0], t[1], R, prec) <= 200 * 1024)
+          cands.push_back(pvsc_tuning{th, 0, 0, 0.f, 1, t[0], t[1], 0});
+    }
+  return cands;
 }
 
 }  // namespace pvsc
@@ -141,14 +210,6 @@ extern "C" int pvsc_autotune_op(pvsc_lattice* lat, int R, int prec, int op, pvsc
   }
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  std::vector<int> vpt_c = {1};
-  if (prec == PVSC_C64 && R >= 2) vpt_c.push_back(2);
-  std::vector<int> zslab_c = {0};
-  const bool march = lat->g.model == PVSC_TI || lat->g.model == PVSC_WSM;  // z-marching sweeps
-  if (march)
-    for (int z : {4, 8, 16, 32, 64})
-      if (z < lat->g.L[2]) zslab_c.push_back(z);
-  const std::vector<int> bps_c = {0, 1, 2};
   auto saved = lat->tuning.find({R, prec});
   const bool had = saved != lat->tuning.end();
   const pvsc_tuning old = had ? saved->second : pvsc_tuning{};
@@ -202,61 +263,7 @@ extern "C" int pvsc_autotune_op(pvsc_lattice* lat, int R, int prec, int op, pvsc
     *ms = best / 3.f;
     return PVSC_OK;
   };
-  // candidate list: z-marching (all shapes), and for TI the flat, prefetching
-  // and shared-memory staged sweeps in a few shapes each
-  std::vector<pvsc_tuning> cands;
-  if (untuned_is_its_own(lat, R, prec)) cands.push_back(kUntuned);
-  for (int vpt : vpt_c) {
-    const int C = R / vpt;
-    for (int th : {64, 128, 256}) {
-      if (th % C != 0 || th < C) continue;
-      for (int bps : bps_c)
-        for (int zs : zslab_c) cands.push_back(pvsc_tuning{th, bps, zs, 0.f, vpt, 0, 0, 0});
-      if (march) cands.push_back(pvsc_tuning{th, 0, 0, 0.f, vpt, 0, 0, 1});  // flat variant
-      if (lat->g.model == PVSC_TI) {
-        // column tiles of this many threads (z-marching, kernel 5)
-        const int tiles5[][2] = {{4, 4}, {8, 4}, {4, 8}, {8, 8}, {16, 4}, {16, 2}, {2, 8}};
-        for (const auto& t : tiles5)
-          if (t[0] * t[1] * C == th) cands.push_back(pvsc_tuning{th, 0, 0, 0.f, vpt, t[0], t[1], 5});
-        // marching along x (lattices with a short z extent)
-        if (lat->g.L[0] > lat->g.L[2]) cands.push_back(pvsc_tuning{th, 0, 0, 0.f, vpt, 0, 0, 6});
-        if (!(prec == PVSC_C64 && vpt == 1 && R > 1)) {
-          for (int zs : {0, 16}) cands.push_back(pvsc_tuning{th, 0, zs, 0.f, vpt, 0, 0, 2});
-          cands.push_back(pvsc_tuning{th, 0, 0, 0.f, vpt, 0, 0, 3});
-        }
-      }
-    }
-  }
-  // TMA-staged plane tiles (kernel 7): z-chunks chosen automatically or a few fixed depths
-  if (tma_sweep_possible(lat, R, prec)) {
-    // the half tiles of the deeper rings (R = 32, 64: slices on the tiles of R = 16)
-    const int deep_y = R == 1 ? 16 : (R == 2 || R == 4) ? 8 : 4, deep_x = R >= 16 ? 8 : (R <= 2 ? 32 : 16);
-    // blocks_per_sm 1: spread the planes over every SM when there are fewer units
-    // than SMs (the same launch otherwise)
-    for (int zs : {0, 16, 32, 64})
-      if (zs == 0 || zs < lat->g.L[2])
-        for (int spread : {0, 1}) {
-          cands.push_back(pvsc_tuning{256, spread, zs, 0.f, 2, 0, 0, kKernelTma});
-          cands.push_back(pvsc_tuning{256, spread, zs, 0.f, 2, deep_x, deep_y, kKernelTma});
-          if (lat->g.model == PVSC_TI)  // the Weyl cells run eight warps only
-            cands.push_back(pvsc_tuning{512, spread, zs, 0.f, 2, 0, 0, kKernelTma});
-        }
-    // the same tiles marching along x, where the z columns are the shorter
-    if (lat->g.L[0] > lat->g.L[2] && tma_xm_possible(lat, R, prec))
-      for (int zs : {0, 32, 64})
-        if (zs == 0 || zs < lat->g.L[0]) {
-          cands.push_back(pvsc_tuning{256, 0, zs, 0.f, 2, 0, 0, kKernelTmaX});
-          if (lat->g.model == PVSC_TI) cands.push_back(pvsc_tuning{256, 0, zs, 0.f, 2, deep_x, deep_y, kKernelTmaX});
-        }
-  }
-  if (lat->g.model == PVSC_TI)
-    for (int th : {128, 256}) {
-      if (th % R) continue;
-      const int tiles[][2] = {{32, 8}, {16, 8}, {16, 4}, {8, 8}, {8, 4}, {4, 4}};
-      for (const auto& t : tiles)
-        if (t[0] * t[1] <= 2 * th && bulk_smem_bytes(t[0], t[1], R, prec) <= 200 * 1024)
-          cands.push_back(pvsc_tuning{th, 0, 0, 0.f, 1, t[0], t[1], 0});
-    }
+  const std::vector<pvsc_tuning> cands = candidates(lat, R, prec, op);
   for (const pvsc_tuning& cand : cands) {
     float ms = 0.f;
     if ((rc = time_one(cand, &ms)) != PVSC_OK) break;
@@ -279,4 +286,15 @@ extern "C" int pvsc_autotune_op(pvsc_lattice* lat, int R, int prec, int op, pvsc
 
 extern "C" int pvsc_autotune(pvsc_lattice* lat, int R, int prec, pvsc_tuning* best, void* stream) {
   return pvsc_autotune_op(lat, R, prec, PVSC_OP_KPM, best, stream);
+}
+
+extern "C" int pvsc_debug_autotune_candidates(const pvsc_lattice* lat, int R, int prec, int op, pvsc_tuning* out,
+                                              int max, int* n) {
+  if (int rc = check_lattice(lat)) return rc;
+  if (!valid_R(R) || (prec != PVSC_C128 && prec != PVSC_C64) || !n || (max > 0 && !out))
+    return set_error(PVSC_ERR_ARG, "bad R, precision or output");
+  const std::vector<pvsc_tuning> c = candidates(lat, R, prec, op);
+  for (int i = 0; i < max && i < (int)c.size(); ++i) out[i] = c[i];
+  *n = (int)c.size();
+  return PVSC_OK;
 }

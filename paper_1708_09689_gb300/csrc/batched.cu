@@ -681,12 +681,13 @@ int pvsc_autotune_batched(pvsc_lattice* const* lats, int n, int R, int prec, con
   const bool had = saved != l0->tuning.end();
   const pvsc_tuning old = had ? saved->second : pvsc_tuning{};
   size_t wmax = 0;
-  // the untuned batch, where its chains are no entry's (some Lx no multiple of 4): threads = 0
+  // the untuned batch, whose chains are no entry's (a kernel 7 entry runs every lattice on the tiles, the
+  // small ones too, and wants Lx a multiple of 4): threads = 0
   auto install = [&](const pvsc_tuning& t) {
     if (t.threads > 0) l0->tuning[{R, prec}] = t; else l0->tuning.erase({R, prec});
   };
   l0->tuning.erase({R, prec});
-  if (!per_lattice_possible(lats, n, R, prec) && chains_default(lats, n, R, prec, batch_shape(l0, R, prec)))
+  if (chains_default(lats, n, R, prec, batch_shape(l0, R, prec)))
     cands.push_back(pvsc_tuning{0, 0, 0, 0.f, 0, 0, 0, PVSC_UNTUNED});
   for (const pvsc_tuning& c : cands) {
     install(c);
