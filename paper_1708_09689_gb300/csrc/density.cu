@@ -37,12 +37,11 @@ constexpr int kDensityChunk = 1024;  // series coefficients staged in shared mem
 // forms the coefficients c_k = g_k sum_r mu_k^r chunk by chunk in shared
 // memory and every thread runs the Chebyshev recurrence T_{k+1} = 2 x T_k - T_{k-1}
 // through them.  Block row y is spectrum y (mu and rho follow one another).  All
-// of it is fp64, two lanes per SM: blocks of 64 threads and all spectra of a
-// call in one launch put it on as many SMs as there are (eight spectra of 1024
-// energies, 256 moments: eight launches of four 256-thread blocks, 375 us, to
-// one of 128 blocks, 24 us).
-constexpr int kDensityThreads = 64;
-__global__ void __launch_bounds__(kDensityThreads) kpm_density_kernel(int R, int M, const double* __restrict__ mu,
+// of it is fp64, two lanes per SM, so all spectra of a call go in one launch
+// (eight spectra of 1024 energies, 256 moments: eight launches of four
+// 256-thread blocks, 375 us, to one of 128 blocks of 64, 24 us), in the blocks
+// that density_threads picks.
+__global__ void __launch_bounds__(256) kpm_density_kernel(int R, int M, const double* __restrict__ mu,
                                                           int kernel, double lambda, double a, double b,
                                                           double scale, int NE,
                                                           const double* __restrict__ E,
@@ -78,6 +77,25 @@ __global__ void __launch_bounds__(kDensityThreads) kpm_density_kernel(int R, int
     }
   }
   if (j < NE) rho[j] = inside ? scale * sum / (M_PI * a * sqrt(1.0 - x * x)) : 0.0;
+}
+
+// Threads per block, 64, 128 or 256.  Every block forms all M coefficients, about 40 + R fp64
+// operations each, for its t energies' 2 t operations a moment: large calls want large blocks, calls of fewer
+// blocks than SMs small ones.  The least of (blocks on the busiest SM) x (40 + R + 2 t).  2048 moments,
+// us on blocks of 64 / 256 / as picked: R = 8: 1024 energies 203 / 310 / 205, 16384 211 / 310 / 182 (128 threads),
+// 65536 661 / 614 / 575 (128), 2^20 10027 / 8221 / 7682; R = 64, 2^18 energies 3523 / 2367 / 2226.
+static int density_threads(int n, int NE, int R, int kernel, int sms) {
+  int best = 64;
+  double least = 1e300;
+  for (int t : {64, 128, 256}) {
+    const int64_t blocks = ((int64_t)NE + t - 1) / t * n;
+    const double cost = (double)((blocks + sms - 1) / sms) * ((kernel == PVSC_KERNEL_NONE ? 2 : 40) + R + 2 * t);
+    if (cost < least) {
+      least = cost;
+      best = t;
+    }
+  }
+  return best;
 }
 
 // psi(k_q, nu) for nk k-points on a lattice of O orbitals per site (TI 4,
@@ -139,8 +157,12 @@ static int kpm_spectra(int n, int R, int M, const double* mu, int kernel, double
   if (int rc = check_ptr(mu, "mu")) return rc;
   if (int rc = check_ptr(E, "E")) return rc;
   if (int rc = check_ptr(rho, "rho")) return rc;
-  const dim3 grid((NE - 1) / kDensityThreads + 1, n);
-  kpm_density_kernel<<<grid, kDensityThreads, 0, st>>>(R, M, mu, kernel, lambda, a, b, scale, NE, E, rho);
+  int dev = 0, sms = 0;
+  PVSC_CUDA_TRY(cudaGetDevice(&dev));
+  PVSC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int threads = density_threads(n, NE, R, kernel, sms);
+  const dim3 grid((NE - 1) / threads + 1, n);
+  kpm_density_kernel<<<grid, threads, 0, st>>>(R, M, mu, kernel, lambda, a, b, scale, NE, E, rho);
   PVSC_CUDA_TRY(cudaGetLastError());
   return PVSC_OK;
 }
