@@ -154,11 +154,16 @@ def _check(rc: int):
         raise PvscError(rc, _lib.pvsc_last_error().decode())
 
 
+# the current stream's handle without a Stream object around it (3 us a call); not public in torch
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream=None):
-    if stream is not None:
-        return ctypes.c_void_p(stream.cuda_stream)
-    # the current stream's handle without a Stream object around it (3 us a call)
-    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    if stream is None:
+        if _raw_stream is not None:
+            return ctypes.c_void_p(_raw_stream(torch.cuda.current_device()))
+        stream = torch.cuda.current_stream()
+    return ctypes.c_void_p(stream.cuda_stream)
 
 
 def _ptr(t: torch.Tensor | None):
