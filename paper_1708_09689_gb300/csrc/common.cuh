@@ -298,8 +298,9 @@ enum AccMode { ACC_NONE = 0, ACC_INIT = 1, ACC_ADD = 2, ACC_FINAL = 4, ACC_X = 8
 // ---------------------------------------------------------------- deterministic dot reduction
 // acc[d][v]: per-thread fp64 partial sums of dot d for vector rc*VPT+v.  Every
 // block reduces them in a fixed order (warp xor tree, then warps in index
-// order) to one value per (d, r), writes its row of `partials`, and the last
-// block to arrive sums the rows in block order and writes the outputs.  The
+// order) to one value per (d, r) and writes its row of `partials`.  The rows are
+// summed in a fixed order by the next sweep of a KPM chain (finish_prev), by
+// sum_rows_kernel, or by the last block of a two-step sweep (finish_dots).  The
 // result is bitwise reproducible for a given launch configuration.
 constexpr int kMaxThreads = 256;
 

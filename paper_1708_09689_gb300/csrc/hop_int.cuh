@@ -12,8 +12,10 @@
 // power of two above the largest input; inputs within six binary places of the largest enter
 // exactly.  The sum of twelve stays below 2^63 and is exact.  The error, at most 12 2^(E - 1081)
 // and typically 2^(E - 1080), is below one rounding of a partial sum of that size in fp64
-// (2^(E - 1076)), of which the fp64 sum makes up to eleven; the conversion rounds once.  Parts with
-// an exponent field outside [128, 1900] (zeros, subnormals, infinities, NaN) are left to the
+// (2^(E - 1076)), of which the fp64 sum makes up to eleven; the conversion rounds once.  This is a bound
+// against the magnitude of the inputs, not against the result: where the large inputs of a part cancel
+// exactly, inputs below 2^-58 of them are lost, which an fp64 sum keeps if it happens to add the
+// cancelling ones first.  Parts with an exponent field outside [128, 1900] (zeros, subnormals, infinities, NaN) are left to the
 // fp64 sum.
 #pragma once
 

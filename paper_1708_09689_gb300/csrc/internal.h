@@ -100,7 +100,7 @@ constexpr int kKernelTiles = 5;
 // TI sweep marching along x instead of z (short z extents)
 constexpr int kKernelXMarch = 6;
 // TI (and Weyl-cell) sweep with TMA-staged z-plane tiles (sweep_tma.cu):
-// complex64, R = 4 .. 64, Lx a multiple of 4
+// complex64, R = 1 .. 64; as a tuning entry Lx a multiple of 4, untuned any Lx
 constexpr int kKernelTma = 7;
 bool tma_sweep_possible(const pvsc_lattice* lat, int R, int prec);  // what a tuning entry may select
 bool tma_sweep_fits(const pvsc_lattice* lat, int R, int prec);      // what the kernel runs: any Lx

@@ -1,8 +1,12 @@
 // Instantiations of the TMA-staged sweep (sweep_tma.cuh) for complex128 TI
-// vectors, the choice of untuned complex128 TI sweeps of large blocks.  A complex128 site of R vectors has the byte layout of a complex64
-// site of 2R vectors, so the tiles, rings and swizzle of layout 2R serve it
-// (R = 16, 32, 64: slices of 8 vectors on the tiles of layout 16); each thread
-// updates one vector of one site, sixteen warps on the large tile.  This
+// vectors, the choice of untuned complex128 TI sweeps of large blocks.  A
+// complex128 site of R vectors has the byte layout of a complex64 site of 2R
+// vectors, so the tiles, rings and swizzle of layout 2R serve it (R = 16, 32,
+// 64: slices of 8 vectors on the tiles of layout 16); each thread updates one
+// vector of one site, sixteen warps on the large tile.  Sixteen warps leave 128
+// registers a thread, and every instantiation spills some of the eight aligned
+// sums and the tile offsets (the R = 8 KPM sweep 164 bytes of stores and 208 of
+// loads); eight warps on the same tile took 995 us where these take 898.  This
 // unit's kernels report copy-wait timeouts in its own error word.
 #include "sweep_tma.cuh"
 
