@@ -174,13 +174,14 @@ __device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
 }
 
 // Bounded wait for the phase of the given parity; false if it ran out or the
-// block is aborting.
-__device__ __forceinline__ bool tma_wait(uint64_t* bar, unsigned parity, volatile int* abort) {
+// block is aborting.  A wait that ran out marks the device word and, where a call reads one of its own, err.
+__device__ __forceinline__ bool tma_wait(uint64_t* bar, unsigned parity, volatile int* abort, int* err) {
   for (unsigned n = 0; n < kTmaWaitLimit; ++n) {
     if (mbar_try_wait(bar, parity)) return true;
     if ((n & 255u) == 255u && *abort) return false;
   }
   atomicExch(&g_tma_sweep_error, 1);
+  if (err != nullptr) atomicExch(err, 1);
   *abort = 1;
   return false;
 }
@@ -338,6 +339,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
   const int G = gridDim.x / SL;  // blocks per slice
   const int c0 = 32 * sl;       // the slice's rows: innermost tensor-map coordinate
   volatile int* abort = &s_abort;
+  int* err = has_dots(FEAT) ? p.err : nullptr;  // of the calls that read one (KPM chains)
   // This block's units, decoded once into a shared table (x0 | y0 << 16, z0 |
   // planes << 16), so that the per-plane copy logic does no division: in the full
   // waves, units u = vb + lu G (lu < nfull) of the slice in wave order (tiles
@@ -572,7 +574,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
       col[i] = XM ? (int64_t)LX * ((x0 + lx) + (int64_t)LY * (y0 + ly)) : (int64_t)(x0 + lx) + (int64_t)Lx * (y0 + ly);
     }
     // plane z0 - 1: x(z-1) of every site into registers
-    if (!tma_wait(&full_x[kx % L::NXS], (kx / L::NXS) & 1, abort)) {
+    if (!tma_wait(&full_x[kx % L::NXS], (kx / L::NXS) & 1, abort, err)) {
       alive = false;
       break;
     }
@@ -589,13 +591,13 @@ __global__ void __launch_bounds__(32 * NW, 1)
     }
     release_x(kx, lu, -1);
     ++kx;
-    if (!tma_wait(&full_x[kx % L::NXS], (kx / L::NXS) & 1, abort)) {
+    if (!tma_wait(&full_x[kx % L::NXS], (kx / L::NXS) & 1, abort, err)) {
       alive = false;
       break;
     }
     for (int j = 0; j < n; ++j) {
-      if (!tma_wait(&full_x[(kx + 1) % L::NXS], ((kx + 1) / L::NXS) & 1, abort) ||
-          !tma_wait(&full_y[ky % L::NYS], (ky / L::NYS) & 1, abort)) {
+      if (!tma_wait(&full_x[(kx + 1) % L::NXS], ((kx + 1) / L::NXS) & 1, abort, err) ||
+          !tma_wait(&full_y[ky % L::NYS], (ky / L::NYS) & 1, abort, err)) {
         alive = false;
         break;
       }
@@ -790,7 +792,6 @@ __global__ void __launch_bounds__(32 * NW, 1)
   }
   __syncthreads();
   if constexpr (has_dots(FEAT)) {
-    if (threadIdx.x == 0 && s_abort && p.err != nullptr) atomicExch(p.err, 1);
     // fixed-order reduction: the warps' partials in index order, then the
     // blocks' rows by the next sweep of a chain or launch_sum_rows (after an abort
     // the values are garbage)
