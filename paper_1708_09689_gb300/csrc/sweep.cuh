@@ -1483,7 +1483,10 @@ __global__ void __launch_bounds__(256) gr_site_sweep(const __grid_constant__ Swe
   const int64_t Nx = p.g.L[0], Ny = p.g.L[1];
   const int R = p.R, rshift = __ffs(R) - 1;
   const int64_t n = 4 * Nx * Ny * R;
-  const double2* __restrict__ X = static_cast<const double2*>(p.x);
+  // plain loads: under programmatic dependent launch this grid is there while the one before still
+  // writes X, which ld.global.nc does not allow (it may be moved ahead of the wait, and may find lines
+  // that an earlier sweep left in L1)
+  const double2* X = static_cast<const double2*>(p.x);
   const double2* Yin = static_cast<const double2*>(p.yin);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += stride) {
@@ -1497,11 +1500,11 @@ __global__ void __launch_bounds__(256) gr_site_sweep(const __grid_constant__ Swe
     const int64_t cy = nu == 0 ? nbr_minus(c, y, Ny, p.g.per[1], Nx) : nbr_plus(c, y, Ny, p.g.per[1], Nx);
     const int64_t cb = end ? cx : c, cd = end ? cy : cx;
     const int oa = nu == 0 ? 1 : nu - 1, ob = nu == 0 ? 1 : (nu == 3 ? 2 : nu + 1), od = (nu == 0 || nu == 2) ? 3 : 0;
-    const double2 xv = __ldg(X + e);
-    const double2 na = __ldg(X + (((4 * c + oa) << rshift) + r));
+    const double2 xv = X[e];
+    const double2 na = X[((4 * c + oa) << rshift) + r];
     double2 nb = make_double2(0.0, 0.0), nd = nb, yi = nb;
-    if (cb >= 0) nb = __ldg(X + (((4 * cb + ob) << rshift) + r));
-    if (cd >= 0) nd = __ldg(X + (((4 * cd + od) << rshift) + r));
+    if (cb >= 0) nb = X[((4 * cb + ob) << rshift) + r];
+    if (cd >= 0) nd = X[((4 * cd + od) << rshift) + r];
     if (Yin != nullptr) yi = Yin[e];
     const double V = site_potential(p.g, s);
     double2 av = make_double2(0.0, 0.0), h = av, wb = av;
