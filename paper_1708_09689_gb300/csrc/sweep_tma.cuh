@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
   const int G = gridDim.x / SL;  // blocks per slice
   const int c0 = 32 * sl;       // the slice's rows: innermost tensor-map coordinate
   volatile int* abort = &s_abort;
-  int* err = has_dots(FEAT) ? p.err : nullptr;  // of the calls that read one (KPM chains)
+  int* err = has_dots(FEAT) && MODEL == PVSC_TI ? p.err : nullptr;  // of the calls that read one (batches)
   // This block's units, decoded once into a shared table (x0 | y0 << 16, z0 |
   // planes << 16), so that the per-plane copy logic does no division: in the full
   // waves, units u = vb + lu G (lu < nfull) of the slice in wave order (tiles
